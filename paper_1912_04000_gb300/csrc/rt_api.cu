@@ -28,7 +28,7 @@ struct rt_ctx {
   int occ_shade = 0;
   // scene
   float4* d_nodes = nullptr;
-  float4* d_nodes4 = nullptr;
+  uint32_t* d_nodes4 = nullptr;  // kNode4Words words per node
   float4* d_nodes8 = nullptr;
   float4* d_nodes4q = nullptr;  // four-wide nodes with 8-bit quantised child boxes (4 float4 each)
   float4* d_tris = nullptr;
@@ -532,13 +532,14 @@ rt_status rt_load_scene(rt_ctx* c, const float* verts, uint32_t n_verts, const u
     float idf, matf, zero = 0.0f;
     std::memcpy(&idf, &t, 4);
     std::memcpy(&matf, &mid, 4);
-    tr[3 * (size_t)i] = make_float4(v[0][0], v[0][1], v[0][2], idf);
-    tr[3 * (size_t)i + 1] = make_float4(v[1][0], v[1][1], v[1][2], matf);
-    tr[3 * (size_t)i + 2] = make_float4(v[2][0], v[2][1], v[2][2], zero);
+    tr[3 * (size_t)i] = make_float4(v[0][0], v[1][0], v[2][0], idf);
+    tr[3 * (size_t)i + 1] = make_float4(v[0][1], v[1][1], v[2][1], matf);
+    tr[3 * (size_t)i + 2] = make_float4(v[0][2], v[1][2], v[2][2], zero);
     nr[i] = make_float4(nrm64[4 * (size_t)t], nrm64[4 * (size_t)t + 1], nrm64[4 * (size_t)t + 2], matf);
   }
   std::vector<float4> nd;
   std::vector<Bvh4Node> b4;
+  std::vector<uint32_t> d4;  // four-wide nodes in device layout (kNode4Words words each)
   std::vector<float4> d8;  // eight-wide nodes in device layout (14 float4 each)
   std::vector<float4> d4q;  // four-wide nodes with 8-bit child boxes (4 float4 each)
   if (!dev_build) {
@@ -551,10 +552,9 @@ rt_status rt_load_scene(rt_ctx* c, const float* verts, uint32_t n_verts, const u
       nd[2 * i] = make_float4(down(b.lo[0]), down(b.lo[1]), down(b.lo[2]), rf);
       nd[2 * i + 1] = make_float4(up(b.hi[0]), up(b.hi[1]), up(b.hi[2]), cf);
     }
-    // four-wide nodes, padded the same way (empty slots keep their +-inf box)
-    // device layout per node: the six plane float4s, then the children packed
-    // as the traversal stack stores them (ref << 3 | count; 0 for an empty
-    // slot, whose box is never entered), then 16 bytes of padding
+    // four-wide nodes, padded the same way (empty slots keep their +-inf box),
+    // the children packed as the traversal stack stores them (ref << 3 |
+    // count; 0 for an empty slot, whose box is never entered)
     collapse_bvh4(bvh, b4, nullptr);
     for (Bvh4Node& n4 : b4)
       for (int i = 0; i < 4; ++i) {
@@ -624,6 +624,27 @@ rt_status rt_load_scene(rt_ctx* c, const float* verts, uint32_t n_verts, const u
       o4[2] = make_float4(w[4], w[5], 0.0f, 0.0f);
       std::memcpy(&o4[3], n4.ref, 16);
     }
+    // the four-wide nodes in the layout the traversal reads: centres and half
+    // extents of the (padded) child boxes, a half extent rounded up so that it
+    // covers the box
+    d4.resize((size_t)kNode4Words * b4.size());
+    for (size_t j = 0; j < b4.size(); ++j) {
+      const Bvh4Node& n4 = b4[j];
+      const float* plo[3] = {n4.lox, n4.loy, n4.loz};
+      const float* phi[3] = {n4.hix, n4.hiy, n4.hiz};
+      float ctr[3][4], ext[3][4];
+      for (int a = 0; a < 3; ++a)
+        for (int i = 0; i < 4; ++i) {
+          ctr[a][i] = 0.0f;
+          ext[a][i] = -1.0f;
+          if (plo[a][i] > phi[a][i]) continue;  // empty slot
+          ctr[a][i] = (float)(0.5 * ((double)plo[a][i] + (double)phi[a][i]));
+          const double h = std::max((double)phi[a][i] - ctr[a][i], (double)ctr[a][i] - plo[a][i]);
+          ext[a][i] = (float)h;
+          if ((double)ext[a][i] < h) ext[a][i] = std::nextafter(ext[a][i], INFINITY);
+        }
+      pack_node4(ctr, ext, n4.ref, &d4[(size_t)kNode4Words * j]);
+    }
     // eight-wide nodes, padded the same way: the plane float4s (per axis lo
     // of children 0-3, 4-7, hi of 0-3, 4-7), then the children packed
     std::vector<Bvh8Node> b8;
@@ -668,8 +689,8 @@ rt_status rt_load_scene(rt_ctx* c, const float* verts, uint32_t n_verts, const u
   CUDA_TRY(c, cudaMalloc(&c->d_nrm, nr.size() * sizeof(float4)));
   if (!dev_build) {
     CUDA_TRY(c, cudaMalloc(&c->d_nodes, nd.size() * sizeof(float4)));
-    CUDA_TRY(c, cudaMalloc(&c->d_nodes4, b4.size() * sizeof(Bvh4Node)));
-    CUDA_TRY(c, cudaMemcpy(c->d_nodes4, b4.data(), b4.size() * sizeof(Bvh4Node), cudaMemcpyHostToDevice));
+    CUDA_TRY(c, cudaMalloc(&c->d_nodes4, d4.size() * sizeof(uint32_t)));
+    CUDA_TRY(c, cudaMemcpy(c->d_nodes4, d4.data(), d4.size() * sizeof(uint32_t), cudaMemcpyHostToDevice));
     CUDA_TRY(c, cudaMalloc(&c->d_nodes4q, d4q.size() * sizeof(float4)));
     CUDA_TRY(c, cudaMemcpy(c->d_nodes4q, d4q.data(), d4q.size() * sizeof(float4), cudaMemcpyHostToDevice));
     CUDA_TRY(c, cudaMalloc(&c->d_nodes8, d8.size() * sizeof(float4)));
@@ -701,7 +722,7 @@ rt_status rt_load_scene(rt_ctx* c, const float* verts, uint32_t n_verts, const u
     if (!e) e = cudaMalloc(&d_tr_in, tr.size() * sizeof(float4));
     if (!e) e = cudaMalloc(&d_nr_in, nr.size() * sizeof(float4));
     if (!e) e = cudaMalloc(&scratch, lbvh_scratch_bytes(n_tris));
-    if (!e) e = cudaMalloc(&c->d_nodes4, n4cap * 8 * sizeof(float4));
+    if (!e) e = cudaMalloc(&c->d_nodes4, n4cap * kNode4Bytes);
     if (!e) e = cudaMemcpy(d_verts, verts, 3 * (size_t)n_verts * sizeof(float), cudaMemcpyHostToDevice);
     if (!e) e = cudaMemcpy(d_idx, tris, 3 * (size_t)n_tris * sizeof(uint32_t), cudaMemcpyHostToDevice);
     if (!e) e = cudaMemcpy(d_tr_in, tr.data(), tr.size() * sizeof(float4), cudaMemcpyHostToDevice);
@@ -716,7 +737,7 @@ rt_status rt_load_scene(rt_ctx* c, const float* verts, uint32_t n_verts, const u
     cudaStream_t bs = c->stream;
     uint32_t* d_counts = nullptr;
     cudaEventRecord(c->ev[0], bs);
-    launch_lbvh(d_verts, d_idx, n_tris, flo, fhi, padf, d_tr_in, d_nr_in, scratch, (float4*)c->d_nodes4,
+    launch_lbvh(d_verts, d_idx, n_tris, flo, fhi, padf, d_tr_in, d_nr_in, scratch, c->d_nodes4,
                 (float4*)c->d_tris, (float4*)c->d_nrm, &d_counts, c->sms, bs);
     cudaEventRecord(c->ev[1], bs);
     uint32_t counts[2] = {0, 0};
@@ -973,10 +994,13 @@ static rt_status render_impl(rt_ctx* c, const rt_camera* cams, uint32_t n_cams, 
   lc.record = o.probe_map_dev != nullptr;
   lc.variant = (int)o.trace_variant;
   lc.leaf_min = o.leaf_batch ? (int)o.leaf_batch : kDefaultLeafBatch;
+  lc.shadow_leaf = o.leaf_batch ? (int)o.leaf_batch : kDefaultShadowLeafBatch;
   lc.sort_rays = o.ray_order == 1;
-  lc.trace_steps = o.trace_steps ? (int)o.trace_steps : kDefaultTraceSteps;
+  // (rounds of at most kMaxSteps steps: the kernels check a ray's step limit between rounds)
+  constexpr uint32_t kMaxSteps = 1024;
+  lc.trace_steps = o.trace_steps ? (int)std::min(o.trace_steps, kMaxSteps) : kDefaultTraceSteps;
   lc.trace_refill = o.trace_refill ? (int)o.trace_refill : kDefaultTraceRefill;
-  lc.shadow_steps = o.shadow_steps ? (int)o.shadow_steps : kDefaultShadowSteps;
+  lc.shadow_steps = o.shadow_steps ? (int)std::min(o.shadow_steps, kMaxSteps) : kDefaultShadowSteps;
   lc.shadow_refill = o.shadow_refill ? (int)o.shadow_refill : kDefaultShadowRefill;
   Probe probe{o.probe_map_dev, o.probe_L_dev, o.probe_sig_dev};
   WaveParams w{};
@@ -1971,6 +1995,7 @@ rt_status rt_render_photons(rt_ctx* c, const rt_camera* cams, uint32_t n_cams, u
   lc.record = o.probe_map_dev != nullptr;
   lc.variant = 0;
   lc.leaf_min = kDefaultLeafBatch;
+  lc.shadow_leaf = kDefaultShadowLeafBatch;
   lc.sort_rays = false;
   lc.trace_steps = kDefaultTraceSteps;
   lc.trace_refill = kDefaultTraceRefill;

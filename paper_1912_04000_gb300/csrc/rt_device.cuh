@@ -115,14 +115,13 @@ __device__ __forceinline__ void thin_sheet(float c, float n, float k, float alph
 // of exactly zero counts as inside.
 // ---------------------------------------------------------------------------
 struct RayW {
-  float3 o;
-  int kx, ky, kz;
+  float ox, oy, oz;  // origin along the axes kx, ky, kz
+  int kx, ky, kz;    // kz the axis of the direction's largest component
   float Sx, Sy, Sz;
 };
 
 __device__ __forceinline__ RayW ray_prep(float3 o, float3 d) {
   RayW r;
-  r.o = o;
   const float ax = fabsf(d.x), ay = fabsf(d.y), az = fabsf(d.z);
   r.kz = (ax > ay) ? (ax > az ? 0 : 2) : (ay > az ? 1 : 2);
   r.kx = r.kz == 2 ? 0 : r.kz + 1;
@@ -133,22 +132,27 @@ __device__ __forceinline__ RayW ray_prep(float3 o, float3 d) {
     r.kx = r.ky;
     r.ky = t;
   }
+  r.ox = comp(o, r.kx);
+  r.oy = comp(o, r.ky);
+  r.oz = comp(o, r.kz);
   r.Sx = __fdiv_rn(comp(d, r.kx), dz);
   r.Sy = __fdiv_rn(comp(d, r.ky), dz);
   r.Sz = __fdiv_rn(1.0f, dz);
   return r;
 }
 
-// returns t (> 0) or -1
-__device__ __forceinline__ float tri_hit(const RayW& r, float3 va, float3 vb, float3 vc) {
-  const float3 A = sub(va, r.o), B = sub(vb, r.o), C = sub(vc, r.o);
-  const float Akz = comp(A, r.kz), Bkz = comp(B, r.kz), Ckz = comp(C, r.kz);
-  const float Ax = __fsub_rn(comp(A, r.kx), __fmul_rn(r.Sx, Akz));
-  const float Ay = __fsub_rn(comp(A, r.ky), __fmul_rn(r.Sy, Akz));
-  const float Bx = __fsub_rn(comp(B, r.kx), __fmul_rn(r.Sx, Bkz));
-  const float By = __fsub_rn(comp(B, r.ky), __fmul_rn(r.Sy, Bkz));
-  const float Cx = __fsub_rn(comp(C, r.kx), __fmul_rn(r.Sx, Ckz));
-  const float Cy = __fsub_rn(comp(C, r.ky), __fmul_rn(r.Sy, Ckz));
+// Hit distance t (> 0) or -1 of the triangle record tr (DevScene::tris): one
+// row per axis with that component of the three vertices, so that the ray's
+// axis order is an order of loads and needs no selects.
+__device__ __forceinline__ float tri_hit(const RayW& r, const float4* tr) {
+  const float4 X = __ldg(tr + r.kx), Y = __ldg(tr + r.ky), Z = __ldg(tr + r.kz);
+  const float Akz = Z.x - r.oz, Bkz = Z.y - r.oz, Ckz = Z.z - r.oz;
+  const float Ax = __fsub_rn(X.x - r.ox, __fmul_rn(r.Sx, Akz));
+  const float Ay = __fsub_rn(Y.x - r.oy, __fmul_rn(r.Sy, Akz));
+  const float Bx = __fsub_rn(X.y - r.ox, __fmul_rn(r.Sx, Bkz));
+  const float By = __fsub_rn(Y.y - r.oy, __fmul_rn(r.Sy, Bkz));
+  const float Cx = __fsub_rn(X.z - r.ox, __fmul_rn(r.Sx, Ckz));
+  const float Cy = __fsub_rn(Y.z - r.oy, __fmul_rn(r.Sy, Ckz));
   const float U = __fsub_rn(__fmul_rn(Cx, By), __fmul_rn(Cy, Bx));
   const float V = __fsub_rn(__fmul_rn(Ax, Cy), __fmul_rn(Ay, Cx));
   const float W = __fsub_rn(__fmul_rn(Bx, Ay), __fmul_rn(By, Ax));
@@ -169,7 +173,7 @@ __device__ __forceinline__ float4 ldg4(const float4* p) { return __ldg(p); }
 
 // Two adjacent float4 (32 bytes, 32-byte aligned) in one read-only 256-bit
 // load (sm_100 and later).
-__device__ __forceinline__ void ldg8(const float4* p, float4& a, float4& b) {
+__device__ __forceinline__ void ldg8(const void* p, float4& a, float4& b) {
   asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
       : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
       : "l"(p));

@@ -24,18 +24,53 @@ constexpr uint32_t kFlagTerm = 1u << 30;     // shadow ray: path ends at this ve
 constexpr uint32_t kFlagGuidedEsc = 1u << 29;  // sun reached by escape counts with MIS weight wesc[pid]
 constexpr uint32_t kMaxWave = 1u << kPidBits;
 
+// Four-wide node on the device: 96 bytes, three sectors of 32.  Per axis the
+// centres of the four child boxes as floats and their half extents as BF16
+// rounded up, child 0 and 2 in the low halves of two words, child 1 and 3 in
+// the high halves -- a high half is read as the float of the whole word, which
+// only widens it; then the children packed as ref << 3 | count:
+//   {cx[4], hx01, hx23, hy01, hy23} {cy[4], hz01, hz23, 0, 0} {cz[4], child[4]}
+// An empty child has a large negative half extent.  Sectors per visit decide
+// the traversal's load on L1 (see trav_interior4).
+constexpr uint32_t kNode4Bytes = 96, kNode4Words = 24;
+constexpr uint32_t kEmptyHalf = 0xFF7Fu;  // BF16 of -3.4e38
+
+// c, h: centre and half extent per axis and child, h < 0 for an empty one.
+__host__ __device__ inline void pack_node4(const float c[3][4], const float h[3][4], const uint32_t child[4],
+                                           uint32_t w[kNode4Words]) {
+  union {
+    float f;
+    uint32_t u;
+  } v;
+  uint32_t b[3][4];
+  for (int a = 0; a < 3; ++a)
+    for (int i = 0; i < 4; ++i) {
+      v.f = c[a][i];
+      w[8 * a + i] = v.u;
+      v.f = h[a][i];
+      b[a][i] = h[a][i] < 0.0f ? kEmptyHalf : (v.u + 0xFFFFu) >> 16;
+    }
+  for (int i = 0; i < 2; ++i) {
+    w[4 + i] = b[0][2 * i] | (b[0][2 * i + 1] << 16);
+    w[6 + i] = b[1][2 * i] | (b[1][2 * i + 1] << 16);
+    w[12 + i] = b[2][2 * i] | (b[2][2 * i + 1] << 16);
+    w[14 + i] = 0u;
+  }
+  for (int i = 0; i < 4; ++i) w[20 + i] = child[i];
+}
+
 // Scene on the device.
 // nodes: 2 float4 per node {lo.xyz, bits(ref)}, {hi.xyz, bits(count)}; node 1
 //   is the root; the children of an interior node sit at an even index pair
 //   (ref, ref + 1), 64-byte aligned; a leaf has count in [1, 7] triangles
 //   starting at triangle ref.
-// tris: 3 float4 per triangle in leaf order {v0, bits(input id)},
-//   {v1, bits(material)}, {v2, 0}.
+// tris: 3 float4 per triangle in leaf order, one per axis: {v0.x, v1.x, v2.x,
+//   bits(input id)}, {v0.y, v1.y, v2.y, bits(material)}, {v0.z, v1.z, v2.z, 0}.
 // nrm: per leaf-order triangle {unit geometric normal (FP64-rounded),
 //   bits(material)}.
 struct DevScene {
   const float4* nodes;   // binary BVH: 2 float4 per node, node 1 the root
-  const float4* nodes4;  // four-wide BVH: 8 float4 per node, node 0 the root
+  const uint32_t* nodes4;  // four-wide BVH: kNode4Words words per node (pack_node4), node 0 the root
   const float4* nodes8;  // eight-wide BVH: 14 float4 per node, node 0 the root (host builds; else null)
   const float4* nodes4q;  // the four-wide BVH with 8-bit child boxes: 4 float4 per node (host builds; else null)
   const float4* tris;
@@ -142,7 +177,7 @@ void launch_scan(uint32_t* data, size_t n, cudaStream_t st);
 constexpr uint32_t kLbvhMaxTris = 1u << 24;
 size_t lbvh_scratch_bytes(uint32_t n);
 void launch_lbvh(const float* verts, const uint32_t* tri, uint32_t n, const float lo[3], const float hi[3], float pad,
-                 const float4* tri_in, const float4* nrm_in, void* scratch, float4* nodes4, float4* tri_out,
+                 const float4* tri_in, const float4* nrm_in, void* scratch, uint32_t* nodes4, float4* tri_out,
                  float4* nrm_out, uint32_t** counts_out, int sms, cudaStream_t st);
 constexpr int kLbvhLevels = 64;
 // Stable LSD radix sort of (key, value) pairs by the low key_bits bits, 8
@@ -209,10 +244,15 @@ struct Probe {
   uint32_t* sig;
 };
 
-// Default traversal loop parameters (set from measurements on a GB300).
-constexpr int kDefaultTraceSteps = 4, kDefaultTraceRefill = 8;
-constexpr int kDefaultShadowSteps = 4, kDefaultShadowRefill = 12;
-constexpr int kDefaultLeafBatch = 24;
+// Default traversal loop parameters, swept on a GB300 (nave 640 x 480 x 81, two
+// samples / 2M-triangle nave, one).  Closest hits: steps 8, leaf batch 16 48.7
+// / 31.8 ms; steps 4, leaf 24 50.0 / 33.3; steps 12, leaf 20 48.7 / 31.8; refill
+// thresholds of 4 to 16 within 1%, 20 13% slower.  Sun rays: steps 8, leaf 26
+// 13.7 / 10.0 ms; steps 4, leaf 24 14.2 / 10.5; steps 8, leaf 16 15.0 / 10.7.
+constexpr int kDefaultTraceSteps = 8, kDefaultTraceRefill = 8;
+constexpr int kDefaultShadowSteps = 8, kDefaultShadowRefill = 12;
+constexpr int kDefaultLeafBatch = 16;
+constexpr int kDefaultShadowLeafBatch = 26;
 
 // Launchers (rt_kernels.cu).
 struct LaunchCfg {
@@ -224,7 +264,8 @@ struct LaunchCfg {
   int variant;  // traversal: 0 = four-wide, leaf batching; binary: 1 = while-while, 2 = node-or-leaf steps,
                 // 3 = leaf batching
   bool sort_rays;  // reorder the vertex >= 2 and sun-ray queues by cell (needs b.rperm)
-  int leaf_min;  // variant 2: lanes waiting at a leaf that start a leaf phase
+  int leaf_min;  // lanes waiting at a leaf that start a leaf phase: closest hits
+  int shadow_leaf;  // ... sun rays
   int trace_steps, trace_refill;    // closest hit: steps between refill checks, refill threshold
   int shadow_steps, shadow_refill;  // sun rays: the same
 };
@@ -241,7 +282,7 @@ void launch_wave(const LaunchCfg& lc, const DevScene& S, const DevSpectra& P, co
                  const PhotonMaps* pm = nullptr);
 // Sorts the children of the n four-wide nodes far-to-near along the sun
 // (the visit order of sun rays).
-void launch_sun_order4(float4* nodes4, uint32_t n, float3 sun, int sms, cudaStream_t st);
+void launch_sun_order4(uint32_t* nodes4, uint32_t n, float3 sun, int sms, cudaStream_t st);
 void launch_l2_probe(const float4* buf, size_t n4, int iters, float* sink, cudaStream_t st, int sms);
 void launch_philox(const uint32_t* ctr, uint32_t* out, uint64_t n, uint32_t k0, uint32_t k1, cudaStream_t st);
 void launch_trace_closest_rays(const DevScene& S, const float* o, const float* d, uint64_t n, float* t,

@@ -17,13 +17,9 @@
 // of a slot are in different waves, which run in sample order.
 #include <algorithm>
 #include <cstdio>
+#include <type_traits>
 
 #include "rt_device.cuh"
-
-// 1: four-wide node boxes read with 256-bit loads
-#ifndef SRT_NODE_LD256
-#define SRT_NODE_LD256 1
-#endif
 
 namespace srt {
 
@@ -141,31 +137,291 @@ __device__ __forceinline__ bool trav_pop(Trav& tv, const uint2* stack, float tma
 }
 
 // ---------------------------------------------------------------------------
-// Four-wide BVH (node = 8 float4: lo.x, hi.x, lo.y, hi.y, lo.z, hi.z of the
-// four children, then the children packed as ref << 3 | count, then padding).  Per axis the ray's direction
-// sign picks the entry plane (lo for a positive direction) and the exit
-// plane, so one slab test per child needs no min/max of the plane pair and an
-// empty child slot (lo = +inf, hi = -inf) is never entered.  The box test
-// rounds as box_t above.
+// Four-wide BVH.  A visit loads the node's three 32-byte sectors (pack_node4).
+// With every lane of a warp at another node, these loads bound the kernel as
+// much as its instructions do (with four sectors per visit the L1's data path
+// was busy in 85% of the cycles, the issue slots in 70%): what counts is how
+// many sectors a visit reads and that the lanes' sectors lie in different
+// banks.  At a node stride of 128 bytes all lanes read the same quarter of
+// their lines and are served one at a time (18 lanes at random nodes in L1: 82
+// cycles per visit of four loads, 44 with the quarters permuted from node to
+// node); the stride of 96 bytes spreads them by itself.  Closest hits of two
+// samples of the 1024 x 768 nave / one of two 1024 x 768 views of the 2M-triangle
+// nave: planes in 128 bytes 171.8 / 106.2 ms, quarters permuted and this loop
+// 138.2 / 87.4, 96 bytes 128.1 / 81.5, loop parameters swept again 125 / 78;
+// sun rays 50.2 / 38.2 -> 36.7 / 29.2.  64-byte nodes on a 15-bit grid gave
+// 136.8 / 89.4 against 140.6 / 89.3 of the 128-byte nodes they were tried
+// against: a decode per plane costs what the sectors save.
+//
+// A slab of centre c and half extent h is crossed from (c - o) / d - h / |d| to
+// (c - o) / d + h / |d|: no entry and exit plane to select by the ray's sign.
 // ---------------------------------------------------------------------------
-template <bool FMA>
-__device__ __forceinline__ void trav_init4(Trav& tv, float3 o, float3 d) {
-  tv.rw = ray_prep(o, d);
-  const float tiny = 1e-20f;
-  tv.inv.x = 1.0f / (fabsf(d.x) > tiny ? d.x : copysignf(tiny, d.x));
-  tv.inv.y = 1.0f / (fabsf(d.y) > tiny ? d.y : copysignf(tiny, d.y));
-  tv.inv.z = 1.0f / (fabsf(d.z) > tiny ? d.z : copysignf(tiny, d.z));
-  tv.oinv = FMA ? make_float3(o.x * tv.inv.x, o.y * tv.inv.y, o.z * tv.inv.z) : o;
-  tv.best_t = INFINITY;
-  tv.best_id = 0xFFFFFFFFu;
-  tv.best_leaf = -1;
-  tv.sp = 0;
-  tv.iter = 0;
-  tv.ref = 0;
-  tv.cnt = 0;
-  tv.oct = (tv.inv.x < 0.0f ? 1u : 0u) | (tv.inv.y < 0.0f ? 2u : 0u) | (tv.inv.z < 0.0f ? 4u : 0u);
+constexpr uint32_t kIdle = 0xFFFFFFFFu;  // Ray4::cur of a lane without work (no leaf: its count would be 7)
+
+struct Ray4 {
+  float3 inv, ainv, oinv;  // 1 / d, |1 / d|, and o / d (FMA box test) or o (any origin)
+  float best_t;
+  int best_leaf;
+  uint32_t cur;  // packed child to visit: ref << 3 | count (count 0: interior node), or kIdle
+  uint32_t iter;
+};
+
+// What a ray needs only at its leaves or its end lies in shared memory, one
+// word per thread and row: the registers it would hold cost resident blocks,
+// and each block more per SM is worth 4-5% of the traversal's time.  Row i of
+// thread t at word i blockDim.x + t behind `base`.
+struct RayRows {
+  uint32_t a;  // shared address of the thread's word in row 0
+  __device__ __forceinline__ explicit RayRows(uint32_t byte_offset) {
+    extern __shared__ __align__(16) unsigned char trav_smem[];
+    a = (uint32_t)__cvta_generic_to_shared(trav_smem) + byte_offset + 4u * threadIdx.x;
+  }
+  __device__ __forceinline__ void put(uint32_t row, uint32_t v) const {
+    asm volatile("st.shared.b32 [%0], %1;" ::"r"(a + 4u * blockDim.x * row), "r"(v) : "memory");
+  }
+  __device__ __forceinline__ void put(uint32_t row, float v) const { put(row, __float_as_uint(v)); }
+  __device__ __forceinline__ uint32_t get(uint32_t row) const {
+    uint32_t v;
+    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(a + 4u * blockDim.x * row) : "memory");
+    return v;
+  }
+  __device__ __forceinline__ float getf(uint32_t row) const { return __uint_as_float(get(row)); }
+  // rows 0-6: the triangle test's form of the ray
+  __device__ __forceinline__ void put(const RayW& w) const {
+    put(0, w.ox);
+    put(1, w.oy);
+    put(2, w.oz);
+    put(3, w.Sx);
+    put(4, w.Sy);
+    put(5, w.Sz);
+    put(6, (uint32_t)(w.kx | (w.ky << 2) | (w.kz << 4)));
+  }
+  __device__ __forceinline__ RayW ray() const {
+    const uint32_t k = get(6);
+    return RayW{getf(0), getf(1), getf(2), (int)(k & 3u), (int)((k >> 2) & 3u), (int)(k >> 4), getf(3), getf(4), getf(5)};
+  }
+};
+constexpr uint32_t kRayRows = 7;
+// rows of a sun ray behind those: direction, contribution, path id and flags
+constexpr uint32_t kRowDir = 7, kRowContrib = 10, kRowBits = 11, kSunRows = 12;
+
+__device__ __forceinline__ float rcp_approx(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float max3f(float a, float b, float c) {
+  float r;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+__device__ __forceinline__ float min3f(float a, float b, float c) {
+  float r;
+  asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
 }
 
+// The reciprocals only bound boxes: their 1 ulp error scales both distances
+// of a slab alike and is covered by the far distance's margin.
+template <bool FMA>
+__device__ __forceinline__ void ray4_init(Ray4& r, const RayRows& rows, float3 o, float3 d) {
+  rows.put(ray_prep(o, d));
+  const float tiny = 1e-20f;
+  r.inv.x = rcp_approx(fabsf(d.x) > tiny ? d.x : copysignf(tiny, d.x));
+  r.inv.y = rcp_approx(fabsf(d.y) > tiny ? d.y : copysignf(tiny, d.y));
+  r.inv.z = rcp_approx(fabsf(d.z) > tiny ? d.z : copysignf(tiny, d.z));
+  r.oinv = FMA ? make_float3(o.x * r.inv.x, o.y * r.inv.y, o.z * r.inv.z) : o;
+  r.ainv = make_float3(fabsf(r.inv.x), fabsf(r.inv.y), fabsf(r.inv.z));
+  r.best_t = INFINITY;
+  r.best_leaf = -1;
+  r.cur = 0u;
+  r.iter = 0;
+}
+
+// Distances at which the ray enters and leaves the slab of centre c and half
+// extent h.  FMA: the rounding of (c - o) / d moves a plane by at most
+// 2^-24 (|o| + |c - o|), within the 2^-22 (max |coordinate| + eps) by which
+// every box is padded, for origins inside the scene bounds.  Otherwise (any
+// origin) from the two planes.
+template <bool FMA>
+__device__ __forceinline__ void slab4(float c, float h, float inv, float ainv, float oinv, float& tn, float& tf) {
+  if (FMA) {
+    const float tc = fmaf(c, inv, -oinv);
+    tn = fmaf(-h, ainv, tc);
+    tf = fmaf(h, ainv, tc);
+  } else {
+    const float t0 = __fmul_rn(__fsub_rn(__fsub_rn(c, h), oinv), inv);
+    const float t1 = __fmul_rn(__fsub_rn(__fadd_rn(c, h), oinv), inv);
+    tn = inv < 0.0f ? t1 : t0;
+    tf = inv < 0.0f ? t0 : t1;
+  }
+}
+
+// Half extents of children 0-3 of one axis from their two words.
+__device__ __forceinline__ float4 halves(float w01, float w23) {
+  return make_float4(__uint_as_float(__float_as_uint(w01) << 16), w01, __uint_as_float(__float_as_uint(w23) << 16), w23);
+}
+
+// Entry distance of a child box, +inf if it is missed or begins past tmax.
+template <bool FMA>
+__device__ __forceinline__ float child4(const Ray4& r, float cx, float hx, float cy, float hy, float cz, float hz,
+                                        float tmax) {
+  float nx, fx, ny, fy, nz, fz;
+  slab4<FMA>(cx, hx, r.inv.x, r.ainv.x, r.oinv.x, nx, fx);
+  slab4<FMA>(cy, hy, r.inv.y, r.ainv.y, r.oinv.y, ny, fy);
+  slab4<FMA>(cz, hz, r.inv.z, r.ainv.z, r.oinv.z, nz, fz);
+  const float tn = max3f(nx, ny, fmaxf(nz, 0.0f));
+  const float tf = min3f(fx, fy, fminf(fz, tmax));
+  return tn <= tf * 1.0000005f ? tn : INFINITY;
+}
+
+__device__ __forceinline__ void cswap(float& ta, uint32_t& pa, float& tb, uint32_t& pb) {
+  const bool sw = tb < ta;
+  const float t = sw ? tb : ta;
+  const uint32_t p = sw ? pb : pa;
+  tb = sw ? ta : tb;
+  pb = sw ? pa : pb;
+  ta = t;
+  pa = p;
+}
+
+// Traversal stack of one lane for closest hits: the upper entries in shared
+// memory (entry j of thread t at column t of row j, so that the lanes of a
+// warp never conflict), the rest, which one ray in a thousand reaches, in a
+// local array.  From local memory alone 16% of the pops came from L2, on the
+// chain between two node visits (nave frame, closest hits: 144.5 ms against
+// 140.6 with the shared rows).  An entry is a child and its entry distance.
+constexpr uint32_t kRows4 = 6;  // shared entries before the bottom ones move to local memory
+constexpr uint32_t kMove4 = 4;  // entries moved at a time
+// Shared memory of a block: the stacks (a node pushes at most three entries
+// past the rows), then the ray rows.
+constexpr uint32_t stack4_bytes(uint32_t block) { return (kRows4 + 3u) * 8u * block; }
+constexpr uint32_t trace4_smem(uint32_t block) { return stack4_bytes(block) + kRayRows * 4u * block; }
+constexpr uint32_t shadow4_smem(uint32_t block) { return kSunRows * 4u * block; }
+
+struct SharedStack {
+  uint32_t top;   // shared address of the first free entry
+  uint32_t deep;  // entries in local memory
+  uint2* local;   // [kStack + kMove4]
+  __device__ __forceinline__ static uint32_t base() {
+    extern __shared__ __align__(16) unsigned char trav_smem[];
+    return (uint32_t)__cvta_generic_to_shared(trav_smem) + 8u * threadIdx.x;
+  }
+  __device__ __forceinline__ static uint32_t row() { return 8u * blockDim.x; }
+  __device__ __forceinline__ void clear() {
+    top = base();
+    deep = 0u;
+  }
+  __device__ __forceinline__ static void put(uint32_t a, uint2 e) {
+    asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(a), "r"(e.x), "r"(e.y) : "memory");
+  }
+  __device__ __forceinline__ static uint2 get(uint32_t a) {
+    uint2 e;
+    asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(e.x), "=r"(e.y) : "r"(a) : "memory");
+    return e;
+  }
+  __device__ __forceinline__ void push(uint32_t p, float t) {
+    put(top, make_uint2(p, __float_as_uint(t)));
+    top += row();
+  }
+  // After a node's pushes: moves the bottom entries to local memory when the
+  // rows are full; false beyond kStack entries.
+  __device__ __forceinline__ bool settle() {
+    if (top <= base() + kRows4 * row()) return true;
+    if (deep + (top - base()) / row() > (uint32_t)kStack) return false;
+    uint32_t a = base();
+    for (uint32_t j = 0; j < kMove4; ++j, a += row()) local[deep++] = get(a);
+    for (; a < top; a += row()) put(a - kMove4 * row(), get(a));
+    top -= kMove4 * row();
+    return true;
+  }
+  // The next entry that begins within tmax, or kIdle when none is left.
+  __device__ __forceinline__ uint32_t pop(float tmax) {
+    for (;;) {
+      if (top == base()) {
+        if (deep == 0u) return kIdle;
+        deep -= kMove4;
+        for (uint32_t j = 0; j < kMove4; ++j, top += row()) put(top, local[deep + j]);
+      }
+      top -= row();
+      const uint2 e = get(top);
+      if (__uint_as_float(e.y) <= tmax) return e.x;
+    }
+  }
+};
+
+// The same for sun rays, whose entries are children alone: a local array.  A
+// sun ray pushes an eighth of what a closest hit does, and the rows cost L1
+// (nave frame, sun rays: 38.1 ms, 40.0 with shared rows).
+struct LocalStack {
+  int sp;
+  uint32_t* local;  // [kStack + 3]
+  __device__ __forceinline__ void clear() { sp = 0; }
+  __device__ __forceinline__ void push(uint32_t p, float) { local[sp++] = p; }
+  __device__ __forceinline__ bool settle() const { return sp <= kStack; }
+  __device__ __forceinline__ uint32_t pop(float) { return sp > 0 ? local[--sp] : kIdle; }
+};
+
+// Interior node r.cur: enters the nearest child that the ray meets and pushes
+// the others; false if it meets none.  Three compare-exchanges find the
+// nearest child and leave the others nearly sorted (59% of the visits of the
+// nave enter one child, 5% more than two: the full order saves 0.4% of the
+// visits and costs two exchanges more in each).  ANY (sun rays, which need
+// every crossed sheet or one opaque hit, in any order): the entered children
+// in slot order, set by k_sun_order4 (farthest along the sun first).
+template <bool FMA, bool COUNT, bool ANY, class ST>
+__device__ __forceinline__ bool interior4(Ray4& r, ST& stack, const DevScene& S, float tmax, uint32_t* status,
+                                          uint32_t& n_nodes) {
+  // cur = ref << 3: node at byte 96 ref = 12 cur
+  const char* nd = (const char*)S.nodes4 + 12u * (size_t)r.cur;
+  float4 cx, cy, cz, a, b, pf;
+  ldg8(nd, cx, a);
+  ldg8(nd + 32, cy, b);
+  ldg8(nd + 64, cz, pf);
+  const float4 hx = halves(a.x, a.y), hy = halves(a.z, a.w), hz = halves(b.x, b.y);
+  if (COUNT) n_nodes += 4;
+  float t0 = child4<FMA>(r, cx.x, hx.x, cy.x, hy.x, cz.x, hz.x, tmax);
+  float t1 = child4<FMA>(r, cx.y, hx.y, cy.y, hy.y, cz.y, hz.y, tmax);
+  float t2 = child4<FMA>(r, cx.z, hx.z, cy.z, hy.z, cz.z, hz.z, tmax);
+  float t3 = child4<FMA>(r, cx.w, hx.w, cy.w, hy.w, cz.w, hz.w, tmax);
+  uint32_t p0 = __float_as_uint(pf.x), p1 = __float_as_uint(pf.y), p2 = __float_as_uint(pf.z),
+           p3 = __float_as_uint(pf.w);
+  if (ANY) {
+    // the entered child of the lowest slot stays in cur, the one before goes up
+    uint32_t cur = kIdle;
+    if (t3 < INFINITY) cur = p3;
+    if (t2 < INFINITY) {
+      if (cur != kIdle) stack.push(cur, 0.0f);
+      cur = p2;
+    }
+    if (t1 < INFINITY) {
+      if (cur != kIdle) stack.push(cur, 0.0f);
+      cur = p1;
+    }
+    if (t0 < INFINITY) {
+      if (cur != kIdle) stack.push(cur, 0.0f);
+      cur = p0;
+    }
+    r.cur = cur;
+  } else {
+    cswap(t0, p0, t1, p1);
+    cswap(t2, p2, t3, p3);
+    cswap(t0, p0, t2, p2);
+    if (t3 < INFINITY) stack.push(p3, t3);
+    if (t1 < INFINITY) stack.push(p1, t1);
+    if (t2 < INFINITY) stack.push(p2, t2);
+    r.cur = t0 < INFINITY ? p0 : kIdle;
+  }
+  if (!stack.settle()) {
+    atomicOr(status, ST_STACK);
+    r.cur = kIdle;
+    stack.clear();
+  }
+  return r.cur != kIdle;
+}
+
+// The wide variants below (8-bit boxes, eight children) test lo and hi planes,
+// the entry and exit plane picked by the ray's direction signs.
 template <bool FMA>
 __device__ __forceinline__ float slab(float plane, float inv, float oinv) {
   // robust mode: oinv holds the origin itself
@@ -182,98 +438,22 @@ __device__ __forceinline__ float child_t(const Trav& tv, float nx, float fx, flo
   return tn <= tf * 1.0000005f ? tn : INFINITY;
 }
 
-__device__ __forceinline__ void cswap(float& ta, uint32_t& pa, float& tb, uint32_t& pb) {
-  const bool sw = tb < ta;
-  const float t = sw ? tb : ta;
-  const uint32_t p = sw ? pb : pa;
-  tb = sw ? ta : tb;
-  pb = sw ? pa : pb;
-  ta = t;
-  pa = p;
-}
-
-// Interior node: test the four children, descend into the nearest entered
-// one and push the others, the nearer ones last (popped first); with ANY
-// (sun rays, which need every crossed sheet or one opaque hit, in any order)
-// visit the entered children in slot order: descend into the first and push
-// the others with the next one on top.  Slot order is set by k_sun_order4
-// (farthest along the sun first).  Returns false if no child is entered.
-template <bool FMA, bool COUNT, bool ANY = false>
-__device__ __forceinline__ bool trav_interior4(Trav& tv, uint2* stack, const DevScene& S, float tmax,
-                                               uint32_t* status, uint32_t& n_nodes) {
-  const float4* nd = S.nodes4 + 8u * tv.ref;
-#if SRT_NODE_LD256
-  // each axis's plane pair in one 256-bit load (4 instead of 7 loads per
-  // node: the kernel is bound by L1 wavefronts of scattered lanes)
-  float4 lx, hx, ly, hy, lz, hz;
-  ldg8(nd, lx, hx);
-  ldg8(nd + 2, ly, hy);
-  ldg8(nd + 4, lz, hz);
-  const bool sx = tv.oct & 1u, sy = tv.oct & 2u, sz = tv.oct & 4u;
-  const float4 nx = sx ? hx : lx, fx = sx ? lx : hx;
-  const float4 ny = sy ? hy : ly, fy = sy ? ly : hy;
-  const float4 nz = sz ? hz : lz, fz = sz ? lz : hz;
-#else
-  const uint32_t ox = tv.oct & 1u, oy = (tv.oct >> 1) & 1u, oz = (tv.oct >> 2) & 1u;
-  const float4 nx = ldg4(nd + ox), fx = ldg4(nd + (ox ^ 1u));
-  const float4 ny = ldg4(nd + 2u + oy), fy = ldg4(nd + 2u + (oy ^ 1u));
-  const float4 nz = ldg4(nd + 4u + oz), fz = ldg4(nd + 4u + (oz ^ 1u));
-#endif
-  const uint4 pk = __ldg((const uint4*)(nd + 6));  // children: ref << 3 | count
-  if (COUNT) n_nodes += 4;
-  float t0 = child_t<FMA>(tv, nx.x, fx.x, ny.x, fy.x, nz.x, fz.x, tmax);
-  float t1 = child_t<FMA>(tv, nx.y, fx.y, ny.y, fy.y, nz.y, fz.y, tmax);
-  float t2 = child_t<FMA>(tv, nx.z, fx.z, ny.z, fy.z, nz.z, fz.z, tmax);
-  float t3 = child_t<FMA>(tv, nx.w, fx.w, ny.w, fy.w, nz.w, fz.w, tmax);
-  uint32_t p0 = pk.x, p1 = pk.y, p2 = pk.z, p3 = pk.w;
-  const int nh = (t0 < INFINITY) + (t1 < INFINITY) + (t2 < INFINITY) + (t3 < INFINITY);
-  if (nh == 0) return false;
-  if (ANY) {
-    if (tv.sp + nh - 1 > kStack) {
-      atomicOr(status, ST_STACK);
-      tv.sp = 0;
-      return false;
-    }
-    const float tt[4] = {t0, t1, t2, t3};
-    const uint32_t pp[4] = {p0, p1, p2, p3};
-    // entered child j >= 1 (in slot order) goes to stack[sp + nh - 1 - j]
-    const int top = tv.sp + nh - 2;
-    int j = -1;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      if (tt[i] < INFINITY) {
-        if (j < 0) {
-          tv.ref = pp[i] >> 3;
-          tv.cnt = pp[i] & 7u;
-        } else {
-          stack[top - j] = make_uint2(pp[i], 0u);
-        }
-        ++j;
-      }
-    }
-    tv.sp += nh - 1;
-    return true;
-  }
-  // sorting network of four (missed children, at +inf, end up last)
-  cswap(t0, p0, t1, p1);
-  cswap(t2, p2, t3, p3);
-  cswap(t0, p0, t2, p2);
-  cswap(t1, p1, t3, p3);
-  cswap(t1, p1, t2, p2);
-  if (tv.sp + nh - 1 > kStack) {
-    atomicOr(status, ST_STACK);
-    tv.sp = 0;
-    return false;
-  }
-  // entries 1 .. nh-1 go to stack[sp + nh - 1 - j] (entry 1 on top)
-  const int top = tv.sp + nh - 2;
-  if (nh > 1) stack[top] = make_uint2(p1, __float_as_uint(t1));
-  if (nh > 2) stack[top - 1] = make_uint2(p2, __float_as_uint(t2));
-  if (nh > 3) stack[top - 2] = make_uint2(p3, __float_as_uint(t3));
-  tv.sp += nh - 1;
-  tv.ref = p0 >> 3;
-  tv.cnt = p0 & 7u;
-  return true;
+template <bool FMA>
+__device__ __forceinline__ void trav_init_wide(Trav& tv, float3 o, float3 d) {
+  tv.rw = ray_prep(o, d);
+  const float tiny = 1e-20f;
+  tv.inv.x = 1.0f / (fabsf(d.x) > tiny ? d.x : copysignf(tiny, d.x));
+  tv.inv.y = 1.0f / (fabsf(d.y) > tiny ? d.y : copysignf(tiny, d.y));
+  tv.inv.z = 1.0f / (fabsf(d.z) > tiny ? d.z : copysignf(tiny, d.z));
+  tv.oinv = FMA ? make_float3(o.x * tv.inv.x, o.y * tv.inv.y, o.z * tv.inv.z) : o;
+  tv.best_t = INFINITY;
+  tv.best_id = 0xFFFFFFFFu;
+  tv.best_leaf = -1;
+  tv.sp = 0;
+  tv.iter = 0;
+  tv.ref = 0;
+  tv.cnt = 0;
+  tv.oct = (tv.inv.x < 0.0f ? 1u : 0u) | (tv.inv.y < 0.0f ? 2u : 0u) | (tv.inv.z < 0.0f ? 4u : 0u);
 }
 
 // ---------------------------------------------------------------------------
@@ -416,18 +596,12 @@ __device__ __forceinline__ bool trav_interior8(Trav& tv, uint2* stack, const Dev
   return true;
 }
 
-template <bool W4, bool FMA, bool COUNT, bool ANY = false>
-__device__ __forceinline__ bool interior_w(Trav& tv, uint2* stack, const DevScene& S, float tmax, uint32_t* status,
-                                           uint32_t& n_nodes) {
-  return W4 ? trav_interior4<FMA, COUNT, ANY>(tv, stack, S, tmax, status, n_nodes)
-            : trav_interior<FMA, COUNT>(tv, stack, S, tmax, status, n_nodes);
-}
-
-// Starts a ray; false if it misses the binary tree's root box.
-template <bool W4, bool FMA>
+// Starts a ray (WIDE: the eight-wide and 8-bit variants); false if it misses
+// the binary tree's root box.
+template <bool WIDE, bool FMA>
 __device__ __forceinline__ bool init_w(Trav& tv, const DevScene& S, float3 o, float3 d) {
-  if (W4) {
-    trav_init4<FMA>(tv, o, d);
+  if (WIDE) {
+    trav_init_wide<FMA>(tv, o, d);
     return true;
   }
   return trav_init<FMA>(tv, S, o, d);
@@ -436,14 +610,33 @@ __device__ __forceinline__ bool init_w(Trav& tv, const DevScene& S, float3 o, fl
 __device__ __forceinline__ void closest_leaf(Trav& tv, const DevScene& S, uint32_t& n_tris, bool count) {
   for (uint32_t t = tv.ref; t < tv.ref + tv.cnt; ++t) {
     const float4* tr = S.tris + 3u * t;
-    const float4 v0 = ldg4(tr), v1 = ldg4(tr + 1), v2 = ldg4(tr + 2);
     if (count) ++n_tris;
-    const float th = tri_hit(tv.rw, f3(v0), f3(v1), f3(v2));
-    const uint32_t id = __float_as_uint(v0.w);
+    const float th = tri_hit(tv.rw, tr);
+    const uint32_t id = __float_as_uint(__ldg(&tr->w));
     if (th > 0.0f && (th < tv.best_t || (th == tv.best_t && id < tv.best_id))) {
       tv.best_t = th;
       tv.best_leaf = (int)t;
       tv.best_id = id;
+    }
+  }
+}
+
+__device__ __forceinline__ uint32_t tri_id(const DevScene& S, uint32_t t) {
+  return __float_as_uint(__ldg(&S.tris[3 * (size_t)t].w));
+}
+
+// The same for Ray4, which reads the ids only on a tie in t.
+__device__ __forceinline__ void closest_leaf4(Ray4& r, const RayRows& rows, const DevScene& S, uint32_t& n_tris,
+                                              bool count) {
+  const RayW w = rows.ray();
+  const uint32_t ref = r.cur >> 3, end = ref + (r.cur & 7u);
+  for (uint32_t t = ref; t < end; ++t) {
+    if (count) ++n_tris;
+    const float th = tri_hit(w, S.tris + 3u * t);
+    if (th > 0.0f && th <= r.best_t &&
+        (th < r.best_t || r.best_leaf < 0 || tri_id(S, t) < tri_id(S, (uint32_t)r.best_leaf))) {
+      r.best_t = th;
+      r.best_leaf = (int)t;
     }
   }
 }
@@ -481,15 +674,15 @@ __device__ __forceinline__ bool closest_step(Trav& tv, uint2* stack, const DevSc
 
 // Sun-ray leaf: product of thin-glass T_s over every crossed sheet; returns
 // true at the first opaque triangle (T = 0, n_glass = 0xFFFFFFFF).
-__device__ __forceinline__ bool shadow_leaf(Trav& tv, const DevScene& S, const DevSpectra& P, float3 d, uint32_t band,
-                                            float& T, uint32_t& ng, uint32_t& n_tris, bool count) {
-  for (uint32_t t = tv.ref; t < tv.ref + tv.cnt; ++t) {
+__device__ __forceinline__ bool shadow_leaf(const RayW& rw, const DevScene& S, const DevSpectra& P, float3 d,
+                                            uint32_t ref, uint32_t cnt, uint32_t band, float& T, uint32_t& ng,
+                                            uint32_t& n_tris, bool count) {
+  for (uint32_t t = ref; t < ref + cnt; ++t) {
     const float4* tr = S.tris + 3u * t;
-    const float4 v0 = ldg4(tr), v1 = ldg4(tr + 1), v2 = ldg4(tr + 2);
     if (count) ++n_tris;
-    const float th = tri_hit(tv.rw, f3(v0), f3(v1), f3(v2));
+    const float th = tri_hit(rw, tr);
     if (th > 0.0f) {
-      const uint32_t mat = __float_as_uint(v1.w);
+      const uint32_t mat = __float_as_uint(__ldg(&tr[1].w));
       if (__ldg(P.mtype + mat) != 1) {
         T = 0.0f;
         ng = 0xFFFFFFFFu;
@@ -507,30 +700,35 @@ __device__ __forceinline__ bool shadow_leaf(Trav& tv, const DevScene& S, const D
   return false;
 }
 
-// Sun-ray leaf for a path that carries bands band0 + q G, q < nv: the
-// product of thin-glass T_s per band.
-__device__ __forceinline__ bool shadow_leaf4(Trav& tv, const DevScene& S, const DevSpectra& P, float3 d,
-                                             uint32_t band0, uint32_t G, uint32_t nv, float (&T)[4], uint32_t& ng,
-                                             uint32_t& n_tris, bool count) {
-  for (uint32_t t = tv.ref; t < tv.ref + tv.cnt; ++t) {
+// Sun-ray leaf of the four-wide kernel: as above, for the one band (NB = 1) or
+// the four bands band + q G (those the path carries) of the ray's path.  The
+// direction and the path are read at a crossed sheet only.
+template <int NB>
+__device__ __forceinline__ bool shadow_leaf4w(const RayRows& rows, const DevScene& S, const DevSpectra& P,
+                                              const WaveParams& w, uint32_t ref, uint32_t cnt, float (&T)[NB],
+                                              uint32_t& ng, uint32_t& n_tris, bool count) {
+  const RayW rw = rows.ray();
+  for (uint32_t t = ref; t < ref + cnt; ++t) {
     const float4* tr = S.tris + 3u * t;
-    const float4 v0 = ldg4(tr), v1 = ldg4(tr + 1), v2 = ldg4(tr + 2);
     if (count) ++n_tris;
-    const float th = tri_hit(tv.rw, f3(v0), f3(v1), f3(v2));
+    const float th = tri_hit(rw, tr);
     if (th > 0.0f) {
-      const uint32_t mat = __float_as_uint(v1.w);
+      const uint32_t mat = __float_as_uint(__ldg(&tr[1].w));
       if (__ldg(P.mtype + mat) != 1) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) T[q] = 0.0f;
+        for (int q = 0; q < NB; ++q) T[q] = 0.0f;
         ng = 0xFFFFFFFFu;
         return true;
       }
       const float4 nr = ldg4(S.nrm + t);
+      const float3 d = make_float3(rows.getf(kRowDir), rows.getf(kRowDir + 1), rows.getf(kRowDir + 2));
       const float c = fabsf(dot(d, f3(nr)));
+      const uint32_t j = path_id(w, rows.get(kRowBits) & kPidMask).j;
+      const uint32_t nv = NB == 4 ? four_band_count(w, j) : 1u;
 #pragma unroll
-      for (uint32_t q = 0; q < 4u; ++q)
+      for (uint32_t q = 0; q < (uint32_t)NB; ++q)
         if (q < nv) {
-          const uint32_t mb = mat * P.n_bands + band0 + q * G;
+          const uint32_t mb = mat * P.n_bands + w.band_first + j + q * w.band_count;
           const float4 m = ldg4(P.mb + mb);
           float Rs, Ts;
           thin_sheet(c, m.x, m.y, __ldg(P.ad + mb), Rs, Ts);
@@ -556,7 +754,7 @@ __device__ __forceinline__ bool shadow_step(Trav& tv, uint2* stack, const DevSce
       if (!trav_interior<FMA, COUNT>(tv, stack, S, INFINITY, status, n_nodes) && !trav_pop(tv, stack, INFINITY))
         return true;
     }
-    if (shadow_leaf(tv, S, P, d, band, T, ng, n_tris, COUNT)) return true;
+    if (shadow_leaf(tv.rw, S, P, d, tv.ref, tv.cnt, band, T, ng, n_tris, COUNT)) return true;
     return !trav_pop(tv, stack, INFINITY);
   }
   if (++tv.iter > cap) {
@@ -566,7 +764,7 @@ __device__ __forceinline__ bool shadow_step(Trav& tv, uint2* stack, const DevSce
   if (tv.cnt == 0u) {
     if (trav_interior<FMA, COUNT>(tv, stack, S, INFINITY, status, n_nodes)) return false;
   } else {
-    if (shadow_leaf(tv, S, P, d, band, T, ng, n_tris, COUNT)) return true;
+    if (shadow_leaf(tv.rw, S, P, d, tv.ref, tv.cnt, band, T, ng, n_tris, COUNT)) return true;
   }
   return !trav_pop(tv, stack, INFINITY);
 }
@@ -575,50 +773,58 @@ __device__ __forceinline__ uint32_t trav_cap(const DevScene& S) {
   return S.iter_cap ? S.iter_cap : 4u * S.n_nodes + 64u;
 }
 
-// Whole-ray helpers for the single-step entry points (any origin).
+// Whole-ray helpers (any origin).
 __device__ __forceinline__ void closest_hit(const DevScene& S, float3 o, float3 d, float& best_t, int& best_leaf,
                                             uint32_t* status) {
-  Trav tv;
-  uint2 stack[kStack];
+  Ray4 r;
+  uint2 local[kStack + kMove4];
+  SharedStack stack;
+  stack.local = local;
+  const RayRows rows(stack4_bytes(blockDim.x));
   uint32_t a = 0, b = 0;
-  trav_init4<false>(tv, o, d);
+  stack.clear();
+  ray4_init<false>(r, rows, o, d);
   const uint32_t cap = trav_cap(S);
-  for (;;) {
-    if (++tv.iter > cap) {
+  while (r.cur != kIdle) {
+    if (++r.iter > cap) {
       atomicOr(status, ST_ITER);
       break;
     }
-    if (tv.cnt == 0u) {
-      if (trav_interior4<false, false>(tv, stack, S, tv.best_t, status, a)) continue;
+    if ((r.cur & 7u) == 0u) {
+      if (interior4<false, false, false>(r, stack, S, r.best_t, status, a)) continue;
     } else {
-      closest_leaf(tv, S, b, false);
+      closest_leaf4(r, rows, S, b, false);
     }
-    if (!trav_pop(tv, stack, tv.best_t)) break;
+    r.cur = stack.pop(r.best_t);
   }
-  best_t = tv.best_t;
-  best_leaf = tv.best_leaf;
+  best_t = r.best_t;
+  best_leaf = r.best_leaf;
 }
 
 __device__ __forceinline__ float shadow_T(const DevScene& S, const DevSpectra& P, float3 o, float3 d, uint32_t band,
                                           uint32_t& n_glass, uint32_t* status) {
-  Trav tv;
-  uint2 stack[kStack];
+  Ray4 r;
+  uint32_t local[kStack + 3];
+  LocalStack stack;
+  stack.local = local;
   uint32_t a = 0, b = 0;
   float T = 1.0f;
   uint32_t ng = 0;
-  trav_init4<false>(tv, o, d);
+  const RayRows rows(0u);
+  stack.clear();
+  ray4_init<false>(r, rows, o, d);
   const uint32_t cap = trav_cap(S);
-  for (;;) {
-    if (++tv.iter > cap) {
+  while (r.cur != kIdle) {
+    if (++r.iter > cap) {
       atomicOr(status, ST_ITER);
       break;
     }
-    if (tv.cnt == 0u) {
-      if (trav_interior4<false, false>(tv, stack, S, INFINITY, status, a)) continue;
-    } else if (shadow_leaf(tv, S, P, d, band, T, ng, b, false)) {
+    if ((r.cur & 7u) == 0u) {
+      if (interior4<false, false, true>(r, stack, S, INFINITY, status, a)) continue;
+    } else if (shadow_leaf(rows.ray(), S, P, d, r.cur >> 3, r.cur & 7u, band, T, ng, b, false)) {
       break;
     }
-    if (!trav_pop(tv, stack, INFINITY)) break;
+    r.cur = stack.pop(INFINITY);
   }
   n_glass = ng;
   return T;
@@ -778,19 +984,11 @@ constexpr uint32_t kNoRay = 0xFFFFFFFFu;
 #define SRT_TRACE_MIN_BLOCKS 8
 #endif
 constexpr int kTraceMaxThreads = 128, kTraceMinBlocks = SRT_TRACE_MIN_BLOCKS;
-// sun-ray kernel: one band per path with the closest-hit kernel's bound
-// (402 / 633 ms against 410 / 645 at bound 9, 56 registers); four bands per
-// path at least 4 blocks of 256 threads' worth (<= 64 registers)
-#ifndef SRT_SHADOW_MIN_BLOCKS
-#define SRT_SHADOW_MIN_BLOCKS 4
-#endif
-constexpr int kShadowMinBlocks = SRT_SHADOW_MIN_BLOCKS;
-#ifndef SRT_SHADOW_SORTED
-constexpr bool kShadowAnyOrder = true;
-#else
-constexpr bool kShadowAnyOrder = false;
-#endif
-
+// four-wide kernels: 9 blocks of 128 per SM (<= 56 registers, none spilled).
+// Two samples of the 1024 x 768 nave / one of two 1024 x 768 views of the
+// 2M-triangle nave, closest hits: 9 blocks 128.1 / 81.5 ms, 10 (48 registers)
+// 130.0 / 82.3; sun rays 36.7 / 29.2, 8 blocks 37.8 / 30.1, 10 36.4 / 29.2.
+constexpr int kTrace4MinBlocks = 9, kShadow4MinBlocks = 9;
 // Persistent traversal loop: a warp refills its idle lanes from the queue
 // once at least `refill` lanes are idle, and each lane with a ray runs up to
 // `steps` traversal steps between refill checks (steps large and refill 32
@@ -800,9 +998,9 @@ constexpr bool kShadowAnyOrder = false;
 // steps; 2: warp-synchronous phases - interior steps for the lanes at an
 // interior node until at least `leaf_min` lanes wait at a leaf (or none can
 // go on), then one leaf step for every waiting lane, so that the costly
-// triangle tests run with most of their lanes busy; 3 (the default, render
-// option trace_variant 0): as 2 over the four-wide BVH; 4 (trace_variant 4):
-// as 2 over the eight-wide BVH.  Modes 0-2 traverse the binary BVH.
+// triangle tests run with most of their lanes busy; 4 and 5 (trace_variant 4,
+// 5): as 2 over the eight-wide BVH and the 8-bit four-wide one.  Modes 0-2
+// traverse the binary BVH; k_trace4 below, the default, the four-wide one.
 template <bool FMA, bool COUNT, int MODE>
 __global__ void __launch_bounds__(kTraceMaxThreads, kTraceMinBlocks) k_trace(DevScene S, const float4* __restrict__ q, float2* __restrict__ hit,
                                                Counters* cnt, uint32_t k, uint32_t cap, Totals* tot,
@@ -831,7 +1029,7 @@ __global__ void __launch_bounds__(kTraceMaxThreads, kTraceMinBlocks) k_trace(Dev
         if (slot < count) {
           const uint32_t ri = perm ? __ldg(perm + slot) : slot;
           const float4 a = __ldcs(q + 2 * ri), b = __ldcs(q + 2 * ri + 1);
-          if (init_w<MODE >= 3, FMA>(tv, S, f3(a), f3(b))) {
+          if (init_w<MODE >= 4, FMA>(tv, S, f3(a), f3(b))) {
             ray = ri;
           } else {
             __stcs(hit + ri, make_float2(-1.0f, __int_as_float(-1)));
@@ -861,7 +1059,7 @@ __global__ void __launch_bounds__(kTraceMaxThreads, kTraceMinBlocks) k_trace(Dev
             done = !trav_pop(tv, stack, tv.best_t);
           } else if (!(MODE == 5   ? trav_interior4q<FMA, COUNT>(tv, stack, S, tv.best_t, status, nn)
                        : MODE == 4 ? trav_interior8<FMA, COUNT>(tv, stack, S, tv.best_t, status, nn)
-                                   : interior_w<MODE == 3, FMA, COUNT>(tv, stack, S, tv.best_t, status, nn))) {
+                                   : trav_interior<FMA, COUNT>(tv, stack, S, tv.best_t, status, nn))) {
             done = !trav_pop(tv, stack, tv.best_t);
           }
         }
@@ -876,6 +1074,86 @@ __global__ void __launch_bounds__(kTraceMaxThreads, kTraceMinBlocks) k_trace(Dev
         done = closest_step<FMA, COUNT, MODE == 1>(tv, stack, S, icap, status, nn, nt);
       if (done) {
         __stcs(hit + ray, make_float2(tv.best_leaf < 0 ? -1.0f : tv.best_t, __int_as_float(tv.best_leaf)));
+        ray = kNoRay;
+      }
+    }
+  }
+  if (COUNT) {
+    atomicAdd(&tot->nodes, (unsigned long long)nn);
+    atomicAdd(&tot->tris, (unsigned long long)nt);
+  }
+}
+
+// Closest hits over the four-wide BVH (render option trace_variant 0):
+// persistent warps refill idle lanes from the queue; a warp runs interior
+// steps for its lanes at interior nodes until at least leaf_min lanes wait at
+// a leaf (or none can go on), then one leaf step for every waiting lane.  The
+// loop's own instructions weigh as much as a box test, so each step takes one
+// vote, and the step limit is checked between rounds of `steps`.
+template <bool FMA, bool COUNT>
+__global__ void __launch_bounds__(kTraceMaxThreads, kTrace4MinBlocks)
+    k_trace4(DevScene S, const float4* __restrict__ q, float2* __restrict__ hit, Counters* cnt, uint32_t k, uint32_t cap,
+             Totals* tot, uint32_t* status, int steps, int refill, int leaf_min, const uint32_t* __restrict__ perm) {
+  const uint32_t count = min(cnt[k].q_count, cap);
+  if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&tot->ext_rays, (unsigned long long)count);
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t lt = (1u << lane) - 1u;
+  const uint32_t icap = trav_cap(S);
+  uint32_t nn = 0, nt = 0;
+  Ray4 r;
+  uint2 local[kStack + kMove4];
+  SharedStack stack;
+  stack.local = local;
+  stack.clear();
+  const RayRows rows(stack4_bytes(blockDim.x));
+  uint32_t ray = kNoRay;
+  r.cur = kIdle;
+  bool drained = count == 0u;
+  for (;;) {
+    const uint32_t idle = __ballot_sync(0xffffffffu, ray == kNoRay);
+    if (!drained && (int)__popc(idle) >= refill) {
+      const uint32_t n = __popc(idle);
+      uint32_t base = 0;
+      if (lane == 0) base = atomicAdd(&cnt[k].q_fetch, n);
+      base = __shfl_sync(0xffffffffu, base, 0);
+      if (base + n >= count) drained = true;
+      const uint32_t slot = base + __popc(idle & lt);
+      if (ray == kNoRay && slot < count) {
+        ray = perm ? __ldg(perm + slot) : slot;
+        const float4 a = __ldcs(q + 2 * ray), b = __ldcs(q + 2 * ray + 1);
+        ray4_init<FMA>(r, rows, f3(a), f3(b));
+      }
+    } else if (idle == 0xffffffffu) {
+      break;  // drained
+    }
+    // a leaf step once all but this many of the lanes with a ray have left
+    // the interior (they wait at a leaf, or have finished in this round)
+    const int nodes_min = (int)__popc(__ballot_sync(0xffffffffu, ray != kNoRay)) - leaf_min;
+    for (int i = 0; i < steps; ++i) {
+      const bool at_node = (r.cur & 7u) == 0u;
+      const bool at_leaf = !at_node && r.cur != kIdle;
+      const uint32_t mi = __ballot_sync(0xffffffffu, at_node);
+      if (mi == 0u || (int)__popc(mi) <= nodes_min) {
+        if (!__any_sync(0xffffffffu, at_leaf)) break;  // none left, or refill first
+        if (at_leaf) {
+          ++r.iter;
+          closest_leaf4(r, rows, S, nt, COUNT);
+          r.cur = stack.pop(r.best_t);
+        }
+      } else if (at_node) {
+        ++r.iter;
+        if (!interior4<FMA, COUNT, false>(r, stack, S, r.best_t, status, nn))
+          r.cur = stack.pop(r.best_t);
+      }
+    }
+    if (ray != kNoRay) {
+      if (r.iter > icap) {
+        atomicOr(status, ST_ITER);
+        r.cur = kIdle;
+        stack.clear();
+      }
+      if (r.cur == kIdle) {
+        __stcs(hit + ray, make_float2(r.best_leaf < 0 ? -1.0f : r.best_t, __int_as_float(r.best_leaf)));
         ray = kNoRay;
       }
     }
@@ -1427,18 +1705,156 @@ __global__ void __launch_bounds__(256, 3) k_shade4(DevScene S, DevSpectra P, Wav
   }
 }
 
-// NB = 4: every sun ray belongs to a path that carries four bands; the ray
-// gathers one transmittance per band and the contributions wait in C4.
-template <bool RECORD, bool COUNT, int MODE, int NB = 1>
-__global__ void __launch_bounds__(NB == 1 ? kTraceMaxThreads : 256, NB == 1 ? kTraceMinBlocks : kShadowMinBlocks)
-    k_shadow(DevScene S, DevSpectra P, WaveParams w, uint32_t k,
-                                                const float4* __restrict__ sq, float* __restrict__ Lbuf,
-                                                uint32_t* __restrict__ sigbuf, Counters* cnt, uint32_t cap,
-                                                double* __restrict__ accum, Probe probe, Totals* tot,
-                                                uint32_t* status, int steps, int refill, float* Lfinal,
-                                                GuideWave gw, int leaf_min, const uint32_t* __restrict__ perm,
-                                                float4* __restrict__ L4, const float4* __restrict__ C4) {
-  static_assert(NB == 1 || (NB == 4 && MODE >= 2), "four-band sun rays use the leaf-batched traversal");
+// The sun ray of path pid is finished: adds its contribution (transmittance T,
+// ng sheets crossed) to the path's radiance and ends the path if it was
+// waiting for it.
+template <bool RECORD>
+__device__ __forceinline__ void sun_ray_done(const DevSpectra& P, const WaveParams& w, uint32_t k, uint32_t bits,
+                                             float contrib, float T, uint32_t ng, bool rec_sun, const GuideWave& gw,
+                                             float* __restrict__ Lbuf, uint32_t* __restrict__ sigbuf,
+                                             double* __restrict__ accum, const Probe& probe, float* Lfinal) {
+  const uint32_t pid = bits & kPidMask;
+  const PathId id = path_id(w, pid);
+  const float Lp = Lbuf[pid] + contrib * T;
+  if (rec_sun && pid % gw.collect == 0u)
+    ((float*)(gw.raw + kRawF4 * ((k - 1u) * gw.slots_per_vertex + pid / gw.collect) + 5u))[0] =
+        T * __ldg(P.sunL + w.band_first + id.j);
+  uint32_t sg = 0;
+  if (RECORD) sg = mix_sig(sigbuf[pid], ng);
+  if (bits & kFlagTerm) {
+    finalize(w, id, Lp, sg, accum, probe, RECORD);
+    if (Lfinal) Lfinal[pid] = Lp;
+  } else {
+    Lbuf[pid] = Lp;
+    if (RECORD) sigbuf[pid] = sg;
+  }
+}
+
+// The same for a path that carries four bands; its contributions wait in C4.
+template <bool RECORD>
+__device__ __forceinline__ void sun_ray_done4(const WaveParams& w, uint32_t bits, const float (&T)[4], uint32_t ng,
+                                              float4* __restrict__ L4, const float4* __restrict__ C4,
+                                              uint32_t* __restrict__ sigbuf, double* __restrict__ accum,
+                                              const Probe& probe) {
+  const uint32_t pid = bits & kPidMask;
+  const float4 c4 = C4[pid], l4 = L4[pid];
+  const float L[4] = {l4.x + c4.x * T[0], l4.y + c4.y * T[1], l4.z + c4.z * T[2], l4.w + c4.w * T[3]};
+  uint32_t sg = 0;
+  if (RECORD) sg = mix_sig(sigbuf[pid], ng);
+  if (bits & kFlagTerm) {
+    finalize4(w, path_id(w, pid), L, sg, accum, probe, RECORD);
+  } else {
+    L4[pid] = make_float4(L[0], L[1], L[2], L[3]);
+    if (RECORD) sigbuf[pid] = sg;
+  }
+}
+
+// Sun rays over the four-wide BVH (trace_variant 0, and 4 and 5, which change
+// the closest-hit traversal only): the loop of k_trace4, ended by the first
+// opaque hit.  NB = 4: every ray belongs to a path that carries four bands
+// and gathers one transmittance per band.
+template <bool RECORD, bool COUNT, int NB>
+__global__ void __launch_bounds__(kTraceMaxThreads, kShadow4MinBlocks)
+    k_shadow4(DevScene S, DevSpectra P, WaveParams w, uint32_t k, const float4* __restrict__ sq,
+              float* __restrict__ Lbuf, uint32_t* __restrict__ sigbuf, Counters* cnt, uint32_t cap,
+              double* __restrict__ accum, Probe probe, Totals* tot, uint32_t* status, int steps, int refill,
+              float* Lfinal, GuideWave gw, int leaf_min, const uint32_t* __restrict__ perm, float4* __restrict__ L4,
+              const float4* __restrict__ C4) {
+  const bool rec_sun = gw.on && gw.collect != 0u && k <= gw.depth && k < w.depth;
+  const uint32_t count = min(cnt[k].s_count, cap);
+  if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&tot->shadow_rays, (unsigned long long)count);
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t lt = (1u << lane) - 1u;
+  const uint32_t icap = trav_cap(S);
+  uint32_t nn = 0, nt = 0;
+  Ray4 r;
+  uint32_t local[kStack + 3];
+  LocalStack stack;
+  stack.local = local;
+  stack.clear();
+  const RayRows rows(0u);
+  uint32_t ray = kNoRay, ng = 0;
+  float T[NB];
+#pragma unroll
+  for (int q = 0; q < NB; ++q) T[q] = 1.0f;
+  r.cur = kIdle;
+  bool drained = count == 0u;
+  for (;;) {
+    const uint32_t idle = __ballot_sync(0xffffffffu, ray == kNoRay);
+    if (!drained && (int)__popc(idle) >= refill) {
+      const uint32_t n = __popc(idle);
+      uint32_t base = 0;
+      if (lane == 0) base = atomicAdd(&cnt[k].s_fetch, n);
+      base = __shfl_sync(0xffffffffu, base, 0);
+      if (base + n >= count) drained = true;
+      const uint32_t slot = base + __popc(idle & lt);
+      if (ray == kNoRay && slot < count) {
+        ray = perm ? __ldg(perm + slot) : slot;
+        const float4 a = __ldcs(sq + 2 * ray), b = __ldcs(sq + 2 * ray + 1);
+        rows.put(kRowBits, a.w);
+        rows.put(kRowContrib, b.w);
+        rows.put(kRowDir, b.x);
+        rows.put(kRowDir + 1, b.y);
+        rows.put(kRowDir + 2, b.z);
+#pragma unroll
+        for (int q = 0; q < NB; ++q) T[q] = 1.0f;
+        ng = 0;
+        ray4_init<true>(r, rows, f3(a), f3(b));
+      }
+    } else if (idle == 0xffffffffu) {
+      break;  // drained
+    }
+    // a leaf step once all but this many of the lanes with a ray have left
+    // the interior (they wait at a leaf, or have finished in this round)
+    const int nodes_min = (int)__popc(__ballot_sync(0xffffffffu, ray != kNoRay)) - leaf_min;
+    for (int i = 0; i < steps; ++i) {
+      const bool at_node = (r.cur & 7u) == 0u;
+      const bool at_leaf = !at_node && r.cur != kIdle;
+      const uint32_t mi = __ballot_sync(0xffffffffu, at_node);
+      if (mi == 0u || (int)__popc(mi) <= nodes_min) {
+        if (!__any_sync(0xffffffffu, at_leaf)) break;  // none left, or refill first
+        if (at_leaf) {
+          ++r.iter;
+          const bool opaque = shadow_leaf4w<NB>(rows, S, P, w, r.cur >> 3, r.cur & 7u, T, ng, nt, COUNT);
+          if (opaque) stack.clear();
+          r.cur = stack.pop(INFINITY);
+        }
+      } else if (at_node) {
+        ++r.iter;
+        if (!interior4<true, COUNT, true>(r, stack, S, INFINITY, status, nn))
+          r.cur = stack.pop(INFINITY);
+      }
+    }
+    if (ray != kNoRay) {
+      if (r.iter > icap) {
+        atomicOr(status, ST_ITER);
+        r.cur = kIdle;
+        stack.clear();
+      }
+      if (r.cur == kIdle) {
+        const uint32_t bits = rows.get(kRowBits);
+        if constexpr (NB == 4)
+          sun_ray_done4<RECORD>(w, bits, T, ng, L4, C4, sigbuf, accum, probe);
+        else
+          sun_ray_done<RECORD>(P, w, k, bits, rows.getf(kRowContrib), T[0], ng, rec_sun, gw, Lbuf, sigbuf, accum, probe,
+                               Lfinal);
+        ray = kNoRay;
+      }
+    }
+  }
+  if (COUNT) {
+    atomicAdd(&tot->snodes, (unsigned long long)nn);
+    atomicAdd(&tot->stris, (unsigned long long)nt);
+  }
+}
+
+// Sun rays over the binary BVH (trace_variant 1-3), MODE as for k_trace.
+template <bool RECORD, bool COUNT, int MODE>
+__global__ void __launch_bounds__(kTraceMaxThreads, kTraceMinBlocks)
+    k_shadow(DevScene S, DevSpectra P, WaveParams w, uint32_t k, const float4* __restrict__ sq,
+             float* __restrict__ Lbuf, uint32_t* __restrict__ sigbuf, Counters* cnt, uint32_t cap,
+             double* __restrict__ accum, Probe probe, Totals* tot, uint32_t* status, int steps, int refill,
+             float* Lfinal, GuideWave gw, int leaf_min, const uint32_t* __restrict__ perm) {
   const bool rec_sun = gw.on && gw.collect != 0u && k <= gw.depth && k < w.depth;
   const uint32_t count = min(cnt[k].s_count, cap);
   if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&tot->shadow_rays, (unsigned long long)count);
@@ -1448,10 +1864,8 @@ __global__ void __launch_bounds__(NB == 1 ? kTraceMaxThreads : 256, NB == 1 ? kT
   uint32_t nn = 0, nt = 0;
   Trav tv;
   uint2 stack[kStack];
-  uint32_t ray = kNoRay, bits = 0, band = 0, ng = 0, nv = 1;
-  float contrib = 0.0f, T[NB];
-#pragma unroll
-  for (int q = 0; q < NB; ++q) T[q] = 1.0f;
+  uint32_t ray = kNoRay, bits = 0, band = 0, ng = 0;
+  float contrib = 0.0f, T = 1.0f;
   float3 dir = make_float3(0.0f, 0.0f, 0.0f);
   bool drained = count == 0u;
   for (;;) {
@@ -1471,13 +1885,10 @@ __global__ void __launch_bounds__(NB == 1 ? kTraceMaxThreads : 256, NB == 1 ? kT
           bits = __float_as_uint(a.w);
           contrib = b.w;
           dir = f3(b);
-          const uint32_t j = path_id(w, bits & kPidMask).j;
-          band = w.band_first + j;
-          if (NB == 4) nv = four_band_count(w, j);
-#pragma unroll
-          for (int q = 0; q < NB; ++q) T[q] = 1.0f;
+          band = w.band_first + path_id(w, bits & kPidMask).j;
+          T = 1.0f;
           ng = 0;
-          if (!init_w<MODE == 3, true>(tv, S, f3(a), dir)) tv.sp = -1;  // misses everything: finished
+          if (!init_w<false, true>(tv, S, f3(a), dir)) tv.sp = -1;  // misses everything: finished
         }
       }
     }
@@ -1500,11 +1911,9 @@ __global__ void __launch_bounds__(NB == 1 ? kTraceMaxThreads : 256, NB == 1 ? kT
             atomicOr(status, ST_ITER);
             done = true;
           } else if (leaf_phase) {
-            bool opaque;
-            if constexpr (NB == 4) opaque = shadow_leaf4(tv, S, P, dir, band, w.band_count, nv, T, ng, nt, COUNT);
-            else opaque = shadow_leaf(tv, S, P, dir, band, T[0], ng, nt, COUNT);
-            done = opaque || !trav_pop(tv, stack, INFINITY);
-          } else if (!interior_w<MODE == 3, true, COUNT, kShadowAnyOrder>(tv, stack, S, INFINITY, status, nn)) {
+            done = shadow_leaf(tv.rw, S, P, dir, tv.ref, tv.cnt, band, T, ng, nt, COUNT) ||
+                   !trav_pop(tv, stack, INFINITY);
+          } else if (!trav_interior<true, COUNT>(tv, stack, S, INFINITY, status, nn)) {
             done = !trav_pop(tv, stack, INFINITY);
           }
         }
@@ -1512,41 +1921,10 @@ __global__ void __launch_bounds__(NB == 1 ? kTraceMaxThreads : 256, NB == 1 ? kT
     } else if (ray != kNoRay) {
       done = tv.sp < 0;
       for (int i = 0; i < steps && !done; ++i)
-        done = shadow_step<true, COUNT, MODE == 1>(tv, stack, S, P, dir, band, T[0], ng, icap, status, nn, nt);
-    }
-    if constexpr (NB == 4) {
-      if (done) {
-        const uint32_t pid = bits & kPidMask;
-        const float4 c4 = C4[pid], l4 = L4[pid];
-        const float L[4] = {l4.x + c4.x * T[0], l4.y + c4.y * T[1], l4.z + c4.z * T[2], l4.w + c4.w * T[3]};
-        uint32_t sg = 0;
-        if (RECORD) sg = mix_sig(sigbuf[pid], ng);
-        if (bits & kFlagTerm) {
-          finalize4(w, path_id(w, pid), L, sg, accum, probe, RECORD);
-        } else {
-          L4[pid] = make_float4(L[0], L[1], L[2], L[3]);
-          if (RECORD) sigbuf[pid] = sg;
-        }
-        ray = kNoRay;
-      }
-      continue;
+        done = shadow_step<true, COUNT, MODE == 1>(tv, stack, S, P, dir, band, T, ng, icap, status, nn, nt);
     }
     if (done) {
-      const uint32_t pid = bits & kPidMask;
-      const PathId id = path_id(w, pid);
-      const float Lp = Lbuf[pid] + contrib * T[0];
-      if (rec_sun && pid % gw.collect == 0u)
-        ((float*)(gw.raw + kRawF4 * ((k - 1u) * gw.slots_per_vertex + pid / gw.collect) + 5u))[0] =
-            T[0] * __ldg(P.sunL + w.band_first + id.j);
-      uint32_t sg = 0;
-      if (RECORD) sg = mix_sig(sigbuf[pid], ng);
-      if (bits & kFlagTerm) {
-        finalize(w, id, Lp, sg, accum, probe, RECORD);
-        if (Lfinal) Lfinal[pid] = Lp;
-      } else {
-        Lbuf[pid] = Lp;
-        if (RECORD) sigbuf[pid] = sg;
-      }
+      sun_ray_done<RECORD>(P, w, k, bits, contrib, T, ng, rec_sun, gw, Lbuf, sigbuf, accum, probe, Lfinal);
       ray = kNoRay;
     }
   }
@@ -1802,56 +2180,77 @@ int grid_for(uint64_t n, int block) {
 }
 
 template <bool FMA, bool COUNT, int MODE>
-void trace_t(const LaunchCfg& lc, const DevScene& S, const float4* qin, const WaveBufs& b, uint32_t k, cudaStream_t st) {
-  const uint32_t* perm = (lc.sort_rays && k >= 2 && b.rperm) ? b.rperm : nullptr;
+void trace_t(const LaunchCfg& lc, const DevScene& S, const float4* qin, const WaveBufs& b, uint32_t k,
+             const uint32_t* perm, cudaStream_t st) {
   k_trace<FMA, COUNT, MODE><<<lc.grid_trace, lc.block_trace, 0, st>>>(S, qin, b.hit, b.cnt, k, b.cap, b.tot, b.status,
                                                                      lc.trace_steps, lc.trace_refill, lc.leaf_min,
                                                                      perm);
 }
 
 template <bool FMA, bool COUNT>
-void trace_m(const LaunchCfg& lc, const DevScene& S, const float4* qin, const WaveBufs& b, uint32_t k,
+void trace4_t(const LaunchCfg& lc, const DevScene& S, const float4* qin, const WaveBufs& b, uint32_t k,
+              const uint32_t* perm, cudaStream_t st) {
+  k_trace4<FMA, COUNT><<<lc.grid_trace, lc.block_trace, trace4_smem(lc.block_trace), st>>>(S, qin, b.hit, b.cnt, k, b.cap, b.tot, b.status,
+                                                                 lc.trace_steps, lc.trace_refill, lc.leaf_min, perm);
+}
+
+template <bool COUNT>
+void trace_m(const LaunchCfg& lc, bool robust, const DevScene& S, const float4* qin, const WaveBufs& b, uint32_t k,
              cudaStream_t st) {
-  if (lc.variant == 5) trace_t<FMA, COUNT, 5>(lc, S, qin, b, k, st);
-  else if (lc.variant == 4) trace_t<FMA, COUNT, 4>(lc, S, qin, b, k, st);
-  else if (lc.variant == 3) trace_t<FMA, COUNT, 2>(lc, S, qin, b, k, st);
-  else if (lc.variant == 2) trace_t<FMA, COUNT, 0>(lc, S, qin, b, k, st);
-  else if (lc.variant == 1) trace_t<FMA, COUNT, 1>(lc, S, qin, b, k, st);
-  else trace_t<FMA, COUNT, 3>(lc, S, qin, b, k, st);
+  const uint32_t* perm = (lc.sort_rays && k >= 2 && b.rperm) ? b.rperm : nullptr;
+  if (lc.variant == 0) {
+    if (robust) trace4_t<false, COUNT>(lc, S, qin, b, k, perm, st);
+    else trace4_t<true, COUNT>(lc, S, qin, b, k, perm, st);
+    return;
+  }
+  auto run = [&](auto fma) {
+    constexpr bool F = decltype(fma)::value;
+    if (lc.variant == 5) trace_t<F, COUNT, 5>(lc, S, qin, b, k, perm, st);
+    else if (lc.variant == 4) trace_t<F, COUNT, 4>(lc, S, qin, b, k, perm, st);
+    else if (lc.variant == 3) trace_t<F, COUNT, 2>(lc, S, qin, b, k, perm, st);
+    else if (lc.variant == 2) trace_t<F, COUNT, 0>(lc, S, qin, b, k, perm, st);
+    else trace_t<F, COUNT, 1>(lc, S, qin, b, k, perm, st);
+  };
+  if (robust) run(std::false_type{});
+  else run(std::true_type{});
 }
 
 void launch_trace(const LaunchCfg& lc, bool robust, const DevScene& S, const float4* qin, const WaveBufs& b, uint32_t k,
                   cudaStream_t st) {
-  if (robust) {
-    if (lc.counting) trace_m<false, true>(lc, S, qin, b, k, st);
-    else trace_m<false, false>(lc, S, qin, b, k, st);
-  } else {
-    if (lc.counting) trace_m<true, true>(lc, S, qin, b, k, st);
-    else trace_m<true, false>(lc, S, qin, b, k, st);
-  }
+  if (lc.counting) trace_m<true>(lc, robust, S, qin, b, k, st);
+  else trace_m<false>(lc, robust, S, qin, b, k, st);
 }
 
-template <bool RECORD, bool COUNT, int MODE, int NB = 1>
+template <bool RECORD, bool COUNT, int MODE>
 void shadow_t(const LaunchCfg& lc, const DevScene& S, const DevSpectra& P, const WaveParams& w, uint32_t k,
               const WaveBufs& b, double* accum, const Probe& probe, float* Lfinal, const GuideWave& gw,
               cudaStream_t st) {
   const uint32_t* perm = (lc.sort_rays && b.rperm) ? b.rperm : nullptr;
-  k_shadow<RECORD, COUNT, MODE, NB><<<lc.grid_shadow, lc.block_trace, 0, st>>>(
+  k_shadow<RECORD, COUNT, MODE><<<lc.grid_shadow, lc.block_trace, 0, st>>>(
       S, P, w, k, b.sq, b.L, b.sig, b.cnt, b.cap, accum, probe, b.tot, b.status, lc.shadow_steps, lc.shadow_refill,
-      Lfinal, gw, lc.leaf_min, perm, b.L4, b.C4);
+      Lfinal, gw, lc.leaf_min, perm);
+}
+
+template <bool RECORD, bool COUNT, int NB>
+void shadow4_t(const LaunchCfg& lc, const DevScene& S, const DevSpectra& P, const WaveParams& w, uint32_t k,
+               const WaveBufs& b, double* accum, const Probe& probe, float* Lfinal, const GuideWave& gw,
+               cudaStream_t st) {
+  const uint32_t* perm = (lc.sort_rays && b.rperm) ? b.rperm : nullptr;
+  k_shadow4<RECORD, COUNT, NB><<<lc.grid_shadow, lc.block_trace, shadow4_smem(lc.block_trace), st>>>(
+      S, P, w, k, b.sq, b.L, b.sig, b.cnt, b.cap, accum, probe, b.tot, b.status, lc.shadow_steps, lc.shadow_refill,
+      Lfinal, gw, lc.shadow_leaf, perm, b.L4, b.C4);
 }
 
 template <bool RECORD, bool COUNT>
 void shadow_m(const LaunchCfg& lc, const DevScene& S, const DevSpectra& P, const WaveParams& w, uint32_t k,
               const WaveBufs& b, double* accum, const Probe& probe, float* Lf, const GuideWave& gw, cudaStream_t st) {
-  // four bands per path: the four-wide tree with leaf batching (the host
-  // refuses other traversal variants there)
-  if (w.nb == 4u) shadow_t<RECORD, COUNT, 3, 4>(lc, S, P, w, k, b, accum, probe, Lf, gw, st);
-  // (the eight-wide variant 4 changes the closest-hit traversal only)
+  // four bands per path: the four-wide tree (the host refuses other traversal
+  // variants there)
+  if (w.nb == 4u) shadow4_t<RECORD, COUNT, 4>(lc, S, P, w, k, b, accum, probe, Lf, gw, st);
   else if (lc.variant == 3) shadow_t<RECORD, COUNT, 2>(lc, S, P, w, k, b, accum, probe, Lf, gw, st);
   else if (lc.variant == 2) shadow_t<RECORD, COUNT, 0>(lc, S, P, w, k, b, accum, probe, Lf, gw, st);
   else if (lc.variant == 1) shadow_t<RECORD, COUNT, 1>(lc, S, P, w, k, b, accum, probe, Lf, gw, st);
-  else shadow_t<RECORD, COUNT, 3>(lc, S, P, w, k, b, accum, probe, Lf, gw, st);
+  else shadow4_t<RECORD, COUNT, 1>(lc, S, P, w, k, b, accum, probe, Lf, gw, st);
 }
 
 void launch_shadow(const LaunchCfg& lc, const DevScene& S, const DevSpectra& P, const WaveParams& w, uint32_t k,
@@ -1885,13 +2284,21 @@ void launch_scan(uint32_t* data, size_t n, cudaStream_t st) {
   k_cell_scan_totals<<<1, (unsigned)(n / 1024u), 0, st>>>(data + n);
 }
 
-void launch_wave(const LaunchCfg& lc, const DevScene& S, const DevSpectra& P, const DevCam* cams, uint32_t n_cams,
+void launch_wave(const LaunchCfg& lcfg, const DevScene& S, const DevSpectra& P, const DevCam* cams, uint32_t n_cams,
                  const WaveParams& w, const WaveBufs& b, double* accum, const Probe& probe, cudaStream_t st,
                  int* launches, StageTimer* tm, const GuideWave* gwp, const GuideDev* gdev, const void* gpack,
                  int sms, const PhotonMaps* pm) {
   GuideWave gw{};
   if (gwp) gw = *gwp;
   const bool guided = gw.on;
+  // no more blocks than the wave has paths for: a queue never holds more, and
+  // a block that finds nothing still costs its start and a fetch (32 x 24 box:
+  // 96 blocks instead of 1368)
+  LaunchCfg lc = lcfg;
+  auto blocks = [&](int block) { return (int)((w.n + (uint32_t)block - 1u) / (uint32_t)block); };
+  lc.grid_trace = std::min(lc.grid_trace, blocks(lc.block_trace));
+  lc.grid_shadow = std::min(lc.grid_shadow, blocks(lc.block_trace));
+  lc.grid_shade = std::min(lc.grid_shade, blocks(lc.block_shade));
   const bool rec = lc.record;
   if (tm) tm->begin(STG_CAMERA, st);
   k_camera<<<grid_for(w.n, 256), 256, 0, st>>>(cams, n_cams, w, b.q[1], b.L, b.sig, b.cnt, rec, b.L4, b.T4, b.cap,
@@ -1963,7 +2370,7 @@ void launch_photon_trace(const DevScene& S, const DevSpectra& P, const PhotonPas
                          uint32_t* vals, uint8_t* cls, uint32_t* status, int sms, cudaStream_t st) {
   const uint64_t n = (uint64_t)pp.Bc * pp.N;
   const unsigned g = (unsigned)std::min<uint64_t>((n + 127) / 128, (uint64_t)(sms > 0 ? sms : 1) * 64);
-  k_photon_trace<<<g, 128, 0, st>>>(S, P, pp, rec, keys, vals, cls, status);
+  k_photon_trace<<<g, 128, trace4_smem(128), st>>>(S, P, pp, rec, keys, vals, cls, status);
 }
 
 void launch_photon_maps(const uint32_t* sorted_keys, const uint32_t* sorted_vals, uint32_t n, const float4* rec,
@@ -1977,13 +2384,13 @@ void launch_philox(const uint32_t* ctr, uint32_t* out, uint64_t n, uint32_t k0, 
 
 void launch_trace_closest_rays(const DevScene& S, const float* o, const float* d, uint64_t n, float* t, int32_t* prim,
                                uint32_t* status, cudaStream_t st) {
-  k_closest_rays<<<grid_for(n, 128), 128, 0, st>>>(S, o, d, n, t, prim, status);
+  k_closest_rays<<<grid_for(n, 128), 128, trace4_smem(128), st>>>(S, o, d, n, t, prim, status);
 }
 
 void launch_trace_shadow_rays(const DevScene& S, const DevSpectra& P, const float* o, const float* d,
                               const uint32_t* band, uint64_t n, float* T, uint32_t* n_glass, uint32_t* status,
                               cudaStream_t st) {
-  k_shadow_rays<<<grid_for(n, 128), 128, 0, st>>>(S, P, o, d, band, n, T, n_glass, status);
+  k_shadow_rays<<<grid_for(n, 128), 128, shadow4_smem(128), st>>>(S, P, o, d, band, n, T, n_glass, status);
 }
 
 void launch_optics(const float* c, const float* n, const float* k, const float* lam, const float* d, uint64_t count,
@@ -2000,19 +2407,19 @@ void launch_optics(const float* c, const float* n, const float* k, const float* 
 // sooner (nave: 5.2 instead of 8.0 node visits per sun ray, counted on the
 // CPU).  Closest-hit traversal sorts children per ray and does not depend
 // on slot order.
-__global__ void k_sun_order4(float4* __restrict__ nodes4, uint32_t n, float3 s) {
+__global__ void k_sun_order4(uint32_t* __restrict__ nodes4, uint32_t n, float3 s) {
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    float* f = reinterpret_cast<float*>(nodes4 + 8 * (size_t)i);
-    float x[28];
+    uint32_t* w = nodes4 + (size_t)kNode4Words * i;
+    uint32_t x[kNode4Words];
 #pragma unroll
-    for (int q = 0; q < 28; ++q) x[q] = f[q];
+    for (uint32_t q = 0; q < kNode4Words; ++q) x[q] = w[q];
     float key[4];
     uint32_t pk[4];
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-      pk[c] = __float_as_uint(x[24 + c]);
+      pk[c] = x[20 + c];
       key[c] = pk[c] == 0u ? -INFINITY
-                           : (x[c] + x[4 + c]) * s.x + (x[8 + c] + x[12 + c]) * s.y + (x[16 + c] + x[20 + c]) * s.z;
+                           : __uint_as_float(x[c]) * s.x + __uint_as_float(x[8 + c]) * s.y + __uint_as_float(x[16 + c]) * s.z;
     }
     int rank[4];
 #pragma unroll
@@ -2024,13 +2431,22 @@ __global__ void k_sun_order4(float4* __restrict__ nodes4, uint32_t n, float3 s) 
       rank[c] = r;
     }
 #pragma unroll
-    for (int q = 0; q < 7; ++q)
+    for (int c = 0; c < 4; ++c) {
 #pragma unroll
-      for (int c = 0; c < 4; ++c) f[4 * q + rank[c]] = x[4 * q + c];
+      for (int a = 0; a < 3; ++a) w[8 * a + rank[c]] = x[8 * a + c];
+      w[20 + rank[c]] = x[20 + c];
+      // half extents: 16-bit halves of words 4-7 (x, y) and 12-13 (z)
+      uint16_t* h = (uint16_t*)w;
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        const int at = a == 2 ? 12 : 4 + 2 * a;
+        h[2 * at + rank[c]] = (uint16_t)(x[at + c / 2] >> (16 * (c & 1)));
+      }
+    }
   }
 }
 
-void launch_sun_order4(float4* nodes4, uint32_t n, float3 sun, int sms, cudaStream_t st) {
+void launch_sun_order4(uint32_t* nodes4, uint32_t n, float3 sun, int sms, cudaStream_t st) {
   if (n == 0) return;
   const uint32_t grid = std::min<uint32_t>((n + 255) / 256, (uint32_t)sms * 8);
   k_sun_order4<<<grid, 256, 0, st>>>(nodes4, n, sun);
@@ -2042,13 +2458,13 @@ void launch_l2_probe(const float4* buf, size_t n4, int iters, float* sink, cudaS
 
 int trace_blocks_per_sm(int block) {
   int a = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_trace<true, false, 3>, block, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_trace4<true, false>, block, trace4_smem(block));
   return a > 0 ? a : 1;
 }
 
 int shadow_blocks_per_sm(int block) {
   int a = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_shadow<false, false, 3>, block, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_shadow4<false, false, 1>, block, shadow4_smem(block));
   return a > 0 ? a : 1;
 }
 

@@ -215,7 +215,7 @@ __device__ __forceinline__ bool small_subtree(const int2* __restrict__ range, in
 
 __global__ void k_lbvh_collapse(int n, const int2* __restrict__ child, const int2* __restrict__ range,
                                 const float4* __restrict__ box, float pad, const int2* __restrict__ qin,
-                                int2* __restrict__ qout, uint32_t* counts, int level, float4* __restrict__ nodes4) {
+                                int2* __restrict__ qout, uint32_t* counts, int level, uint32_t* __restrict__ nodes4) {
   const uint32_t m = counts[1 + level];
   for (uint32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < m; e += gridDim.x * blockDim.x) {
     const int2 item = qin[e];
@@ -243,18 +243,19 @@ __global__ void k_lbvh_collapse(int n, const int2* __restrict__ child, const int
         ch[nc++] = cc.y;
       }
     }
-    float lo[3][4], hi[3][4];
+    float ctr[3][4], ext[3][4];  // centre and half extent of the padded child boxes
     uint32_t pk[4];
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       if (c < nc) {
         const float4 l = __ldcg(box + 2 * ch[c]), h = __ldcg(box + 2 * ch[c] + 1);
-        lo[0][c] = __fsub_rd(l.x, pad);
-        lo[1][c] = __fsub_rd(l.y, pad);
-        lo[2][c] = __fsub_rd(l.z, pad);
-        hi[0][c] = __fadd_ru(h.x, pad);
-        hi[1][c] = __fadd_ru(h.y, pad);
-        hi[2][c] = __fadd_ru(h.z, pad);
+        const float lo[3] = {__fsub_rd(l.x, pad), __fsub_rd(l.y, pad), __fsub_rd(l.z, pad)};
+        const float hi[3] = {__fadd_ru(h.x, pad), __fadd_ru(h.y, pad), __fadd_ru(h.z, pad)};
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          ctr[a][c] = 0.5f * lo[a] + 0.5f * hi[a];
+          ext[a][c] = fmaxf(__fsub_ru(hi[a], ctr[a][c]), __fsub_ru(ctr[a][c], lo[a]));
+        }
         if (ch[c] >= n - 1) {
           pk[c] = ((uint32_t)(ch[c] - (n - 1)) << 3) | 1u;
         } else if (small_subtree(range, n, ch[c])) {
@@ -266,21 +267,16 @@ __global__ void k_lbvh_collapse(int n, const int2* __restrict__ child, const int
           qout[atomicAdd(counts + 2 + level, 1u)] = make_int2(ch[c], (int)slot);
         }
       } else {
-        lo[0][c] = lo[1][c] = lo[2][c] = INFINITY;
-        hi[0][c] = hi[1][c] = hi[2][c] = -INFINITY;
+        ctr[0][c] = ctr[1][c] = ctr[2][c] = 0.0f;
+        ext[0][c] = ext[1][c] = ext[2][c] = -1.0f;
         pk[c] = 0u;
       }
     }
-    float4* o = nodes4 + 8 * (size_t)item.y;
-    o[0] = make_float4(lo[0][0], lo[0][1], lo[0][2], lo[0][3]);
-    o[1] = make_float4(hi[0][0], hi[0][1], hi[0][2], hi[0][3]);
-    o[2] = make_float4(lo[1][0], lo[1][1], lo[1][2], lo[1][3]);
-    o[3] = make_float4(hi[1][0], hi[1][1], hi[1][2], hi[1][3]);
-    o[4] = make_float4(lo[2][0], lo[2][1], lo[2][2], lo[2][3]);
-    o[5] = make_float4(hi[2][0], hi[2][1], hi[2][2], hi[2][3]);
-    o[6] = make_float4(__uint_as_float(pk[0]), __uint_as_float(pk[1]), __uint_as_float(pk[2]),
-                       __uint_as_float(pk[3]));
-    o[7] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    uint32_t w[kNode4Words];
+    pack_node4(ctr, ext, pk, w);
+    uint32_t* o = nodes4 + (size_t)kNode4Words * item.y;
+#pragma unroll
+    for (uint32_t q = 0; q < kNode4Words; ++q) o[q] = w[q];
   }
 }
 
@@ -352,7 +348,7 @@ size_t lbvh_scratch_bytes(uint32_t n) {
 // each collapse level}: a non-zero last entry means the tree was deeper than
 // the levels launched.
 void launch_lbvh(const float* verts, const uint32_t* tri, uint32_t n, const float lo[3], const float hi[3], float pad,
-                 const float4* tri_in, const float4* nrm_in, void* scratch, float4* nodes4, float4* tri_out,
+                 const float4* tri_in, const float4* nrm_in, void* scratch, uint32_t* nodes4, float4* tri_out,
                  float4* nrm_out, uint32_t** counts_out, int sms, cudaStream_t st) {
   const uint32_t nb = (n + kSortTile - 1) / kSortTile;
   const size_t hist_n = ((size_t)256 * nb + 32767) / 32768 * 32768;
