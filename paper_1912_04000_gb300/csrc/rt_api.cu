@@ -965,8 +965,11 @@ static rt_status render_impl(rt_ctx* c, const rt_camera* cams, uint32_t n_cams, 
   cudaStream_t st = c->stream;
   const uint32_t PB = (uint32_t)PB64;
   uint32_t cap = o.wave_capacity ? o.wave_capacity : (1u << 23);
-  cap = std::min<uint32_t>(std::min<uint32_t>(cap, kMaxWave), PB);
-  cap = std::max<uint32_t>(cap, 1u);
+  cap = std::max<uint32_t>(std::min<uint32_t>(cap, kMaxWave), 1u);
+  // several whole samples per wave where they fit; not where paths keep
+  // training slots, whose waves are the batches the guide is trained on
+  const uint32_t m_samples = o.guided && o.guide_collect ? 1u : wave_samples(cap, PB, spp);
+  cap = m_samples > 1 ? m_samples * PB : std::min<uint32_t>(cap, PB);
   if (rt_status e = ensure_wave(c, cap)) return e;
   if (nb == 4)
     if (rt_status e = ensure_four_band(c, cap)) return e;
@@ -1105,10 +1108,15 @@ static rt_status render_impl(rt_ctx* c, const rt_camera* cams, uint32_t n_cams, 
       w.n = (uint32_t)std::min<uint64_t>(cap, total - ws);
       w.s0 = o.sample_first + (uint32_t)(ws / PB);
       w.r0 = (uint32_t)(ws % PB);
+      w.samples = m_samples > 1 ? w.n / PB : 1u;
       if ((e = cudaMemsetAsync(c->wb.cnt, 0, sizeof(Counters) * (depth + 2), s))) return e;
       if (gw.collect && (e = cudaMemsetAsync(gw.raw, 0, (size_t)n_slots * kRawF4 * sizeof(float4), s))) return e;
       launch_wave(lc, S, c->sp, c->d_cams, n_cams, w, wb, accum, probe, s, &launches, tm, &gw, &c->guide.dev,
                   c->guide.pack, c->sms);
+      if (w.samples > 1) {
+        launch_resolve(w, wb, accum, c->sms, s);
+        ++launches;
+      }
       if (o.guide_records_dev) {
         // the wave's records in path order: slot (v, p) -> records 2 (v spv + p) and + 1, copied to
         // path ws + p of vertex v
@@ -1982,8 +1990,16 @@ rt_status rt_render_photons(rt_ctx* c, const rt_camera* cams, uint32_t n_cams, u
   // hit, shading that ends at the first Lambertian vertex, sun rays), one
   // band chunk at a time, into the chunk's columns of the spectral image
   const Probe probe{o.probe_map_dev, o.probe_L_dev, o.probe_sig_dev};
-  uint32_t cap = (uint32_t)std::min<uint64_t>(std::min<uint64_t>(1u << 23, npix * Bc), kMaxWave);
-  cap = std::max<uint32_t>(cap, 1u);
+  // (whole samples per wave where several fit, as in rt_render; the last
+  // chunk's bands may be fewer and its samples smaller)
+  constexpr uint64_t kPhotonWave = 1u << 23;
+  static_assert(kPhotonWave <= kMaxWave, "wave capacity");
+  const uint32_t bc_last = band_count % Bc ? band_count % Bc : Bc;
+  auto wave_of = [&](uint64_t bc) {
+    const uint64_t pb = npix * bc;
+    return std::max<uint64_t>(1, std::min(kPhotonWave, pb * wave_samples(kPhotonWave, pb, spp)));
+  };
+  const uint32_t cap = (uint32_t)std::max(wave_of(Bc), wave_of(bc_last));
   if (rt_status e = ensure_wave(c, cap)) return e;
   LaunchCfg lc;
   lc.block_trace = 128;
@@ -2047,17 +2063,21 @@ rt_status rt_render_photons(rt_ctx* c, const rt_camera* cams, uint32_t n_cams, u
     w.B = bc;
     w.acc_off = cb - band_first;
     w.PB = (uint32_t)(npix * bc);
-    // a wave holds at most one sample's paths of this chunk, so that it
-    // spans two samples at most (path ids wrap once)
-    const uint32_t wcap = std::min<uint32_t>(cap, w.PB);
+    // a wave holds whole samples of this chunk, or a part of one
+    const uint32_t wcap = (uint32_t)wave_of(bc);
     const uint64_t total = (uint64_t)w.PB * spp;
     for (uint64_t ws = 0; ws < total; ws += wcap) {
       w.n = (uint32_t)std::min<uint64_t>(wcap, total - ws);
       w.s0 = (uint32_t)(ws / w.PB);
       w.r0 = (uint32_t)(ws % w.PB);
+      w.samples = wcap > w.PB ? w.n / w.PB : 1u;
       CUDA_TRY(c, cudaMemsetAsync(c->wb.cnt, 0, sizeof(Counters) * (depth + 2), st));
       launch_wave(lc, S, c->sp, c->d_cams, n_cams, w, c->wb, accum, probe, st, &launches, nullptr, nullptr, nullptr,
                   nullptr, c->sms, &M);
+      if (w.samples > 1) {
+        launch_resolve(w, c->wb, accum, c->sms, st);
+        ++launches;
+      }
     }
     mark();
     launches += 1 + 16 + 1;  // photon trace, 4 radix passes of 4 kernels, ranges

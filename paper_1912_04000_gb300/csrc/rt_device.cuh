@@ -202,17 +202,21 @@ __device__ __forceinline__ PathId path_id(const WaveParams& w, uint32_t pid) {
   p.r = w.r0 + pid;
   p.s = w.s0;
   if (p.r >= w.PB) {
-    p.r -= w.PB;
-    p.s += 1;
+    const uint32_t q = p.r / w.PB;
+    p.r -= q * w.PB;
+    p.s += q;
   }
   p.pix = p.r / w.band_count;
   p.j = p.r - p.pix * w.band_count;
   return p;
 }
 
-__device__ __forceinline__ void finalize(const WaveParams& w, const PathId& id, float L, uint32_t sg, double* accum,
-                                         const Probe& probe, bool record) {
-  if (L != 0.0f) accum[(size_t)id.pix * w.acc_stride + w.acc_off + id.j] += (double)L;
+// Termination of path pid: its radiance goes to the image, or in a wave of
+// several samples to its slot of Lbuf.
+__device__ __forceinline__ void finalize(const WaveParams& w, const PathId& id, uint32_t pid, float L, uint32_t sg,
+                                         float* Lbuf, double* accum, const Probe& probe, bool record) {
+  if (w.samples > 1u) Lbuf[pid] = L;
+  else if (L != 0.0f) accum[(size_t)id.pix * w.acc_stride + w.acc_off + id.j] += (double)L;
   if (record && probe.map != nullptr) {
     const uint32_t slot = probe.map[id.pix];
     if (slot != 0xFFFFFFFFu) {
@@ -231,14 +235,18 @@ __device__ __forceinline__ uint32_t four_band_count(const WaveParams& w, uint32_
 
 // Termination of a path that carries four bands: each existing band adds
 // its radiance to its own (pixel, band) slot, as four one-band paths would.
-__device__ __forceinline__ void finalize4(const WaveParams& w, const PathId& id, const float (&L)[4], uint32_t sg,
-                                          double* accum, const Probe& probe, bool record) {
+__device__ __forceinline__ void finalize4(const WaveParams& w, const PathId& id, uint32_t pid, const float (&L)[4],
+                                          uint32_t sg, float4* L4, double* accum, const Probe& probe, bool record) {
   const uint32_t G = w.band_count;
   const uint32_t nv = four_band_count(w, id.j);
   const size_t base = (size_t)id.pix * w.B + id.j;
+  if (w.samples > 1u) {
+    L4[pid] = make_float4(L[0], L[1], L[2], L[3]);
+  } else {
 #pragma unroll
-  for (uint32_t q = 0; q < 4u; ++q)
-    if (q < nv && L[q] != 0.0f) accum[base + q * G] += (double)L[q];
+    for (uint32_t q = 0; q < 4u; ++q)
+      if (q < nv && L[q] != 0.0f) accum[base + q * G] += (double)L[q];
+  }
   if (record && probe.map != nullptr) {
     const uint32_t slot = probe.map[id.pix];
     if (slot != 0xFFFFFFFFu) {

@@ -1102,7 +1102,7 @@ __global__ void __launch_bounds__(kSampleThreads, kSampleCtasPerSm)
           t->w = __uint_as_float(__float_as_uint(t->w) | kFlagTerm);
         } else {
           const float Lp = Lbuf[pid];
-          finalize(w, id, Lp, record ? sigbuf[pid] : 0u, accum, probe, record);
+          finalize(w, id, pid, Lp, record ? sigbuf[pid] : 0u, Lbuf, accum, probe, record);
           if (gw.Lfinal) gw.Lfinal[pid] = Lp;
         }
       }

@@ -129,6 +129,11 @@ struct WaveParams {
   // chunk of a wider spectral image; acc_stride = band_count, acc_off = 0
   // for a whole render)
   uint32_t acc_stride, acc_off;
+  // samples > 1: the wave holds that many whole samples (r0 = 0, n = samples
+  // PB); a path that ends leaves its radiance in its L (L4) slot and
+  // launch_resolve adds the samples to the image in order.  Otherwise the
+  // paths of a slot are in different waves and add to the image themselves.
+  uint32_t samples;
 };
 
 // Guided sampling of one wave (on == false: plain cosine sampling).
@@ -280,6 +285,15 @@ void launch_wave(const LaunchCfg& lc, const DevScene& S, const DevSpectra& P, co
                  cudaStream_t st, int* launches, StageTimer* timer, const GuideWave* gw = nullptr,
                  const GuideDev* gdev = nullptr, const void* gpack = nullptr, int sms = 0,
                  const PhotonMaps* pm = nullptr);
+// Adds a multi-sample wave's radiances to the spectral image, samples in order.
+void launch_resolve(const WaveParams& w, const WaveBufs& b, double* accum, int sms, cudaStream_t st);
+// Samples per wave for PB paths per sample: as many whole samples as the
+// capacity holds (at most spp), else 1.  A render whose samples are far
+// smaller than a wave is bound by the launches and the tails of its waves.
+inline uint32_t wave_samples(uint64_t capacity, uint64_t PB, uint32_t spp) {
+  const uint64_t m = capacity / PB;
+  return (uint32_t)(m < 1 ? 1 : (m > spp ? spp : m));
+}
 // Sorts the children of the n four-wide nodes far-to-near along the sun
 // (the visit order of sun rays).
 void launch_sun_order4(uint32_t* nodes4, uint32_t n, float3 sun, int sms, cudaStream_t st);

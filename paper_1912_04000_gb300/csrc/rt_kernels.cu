@@ -1378,7 +1378,7 @@ __global__ void __launch_bounds__(256, SRT_SHADE_MIN_BLOCKS) k_shade(DevScene S,
         }
       }
       if (terminate && !emit_shadow) {
-        finalize(w, id, Lp, sg, accum, probe, RECORD);
+        finalize(w, id, pid, Lp, sg, Lbuf, accum, probe, RECORD);
         if (GUIDED && gw.Lfinal) gw.Lfinal[pid] = Lp;
       } else {
         Lbuf[pid] = Lp;
@@ -1677,7 +1677,7 @@ __global__ void __launch_bounds__(256, 3) k_shade4(DevScene S, DevSpectra P, Wav
         }
       }
       if (terminate && !emit_shadow) {
-        finalize4(w, id, L, sg, accum, probe, RECORD);
+        finalize4(w, id, pid, L, sg, L4, accum, probe, RECORD);
       } else {
         L4[pid] = make_float4(L[0], L[1], L[2], L[3]);
         if (RECORD) sigbuf[pid] = sg;
@@ -1722,7 +1722,7 @@ __device__ __forceinline__ void sun_ray_done(const DevSpectra& P, const WavePara
   uint32_t sg = 0;
   if (RECORD) sg = mix_sig(sigbuf[pid], ng);
   if (bits & kFlagTerm) {
-    finalize(w, id, Lp, sg, accum, probe, RECORD);
+    finalize(w, id, pid, Lp, sg, Lbuf, accum, probe, RECORD);
     if (Lfinal) Lfinal[pid] = Lp;
   } else {
     Lbuf[pid] = Lp;
@@ -1742,7 +1742,7 @@ __device__ __forceinline__ void sun_ray_done4(const WaveParams& w, uint32_t bits
   uint32_t sg = 0;
   if (RECORD) sg = mix_sig(sigbuf[pid], ng);
   if (bits & kFlagTerm) {
-    finalize4(w, path_id(w, pid), L, sg, accum, probe, RECORD);
+    finalize4(w, path_id(w, pid), pid, L, sg, L4, accum, probe, RECORD);
   } else {
     L4[pid] = make_float4(L[0], L[1], L[2], L[3]);
     if (RECORD) sigbuf[pid] = sg;
@@ -1931,6 +1931,36 @@ __global__ void __launch_bounds__(kTraceMaxThreads, kTraceMinBlocks)
   if (COUNT) {
     atomicAdd(&tot->snodes, (unsigned long long)nn);
     atomicAdd(&tot->stris, (unsigned long long)nt);
+  }
+}
+
+// The image's slots of one wave of whole samples: each takes its paths'
+// radiances in sample order, the order and the sums of one-sample waves.
+// Bound by HBM (4 bytes read per path, 16 moved per slot).
+__global__ void __launch_bounds__(256) k_resolve(WaveParams w, const float* __restrict__ L,
+                                                 const float4* __restrict__ L4, double* __restrict__ accum) {
+  for (uint32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < w.PB; r += gridDim.x * blockDim.x) {
+    const uint32_t pix = r / w.band_count, j = r - pix * w.band_count;
+    if (w.nb == 4u) {
+      const uint32_t nv = four_band_count(w, j);
+      double* a = accum + (size_t)pix * w.B + j;
+      for (uint32_t q = 0; q < nv; ++q) {
+        double v = a[q * w.band_count];
+        for (uint32_t s = 0; s < w.samples; ++s) {
+          const float x = ((const float*)(L4 + (size_t)s * w.PB + r))[q];
+          if (x != 0.0f) v += (double)x;
+        }
+        a[q * w.band_count] = v;
+      }
+    } else {
+      double* a = accum + (size_t)pix * w.acc_stride + w.acc_off + j;
+      double v = *a;
+      for (uint32_t s = 0; s < w.samples; ++s) {
+        const float x = L[(size_t)s * w.PB + r];
+        if (x != 0.0f) v += (double)x;
+      }
+      *a = v;
+    }
   }
 }
 
@@ -2364,6 +2394,11 @@ void launch_wave(const LaunchCfg& lcfg, const DevScene& S, const DevSpectra& P, 
     nl += 3;
   }
   if (launches) *launches += nl;
+}
+
+void launch_resolve(const WaveParams& w, const WaveBufs& b, double* accum, int sms, cudaStream_t st) {
+  const uint32_t g = std::min<uint32_t>((w.PB + 255u) / 256u, (uint32_t)(sms > 0 ? sms : 1) * 16u);
+  k_resolve<<<g, 256, 0, st>>>(w, b.L, b.L4, accum);
 }
 
 void launch_photon_trace(const DevScene& S, const DevSpectra& P, const PhotonPass& pp, float4* rec, uint32_t* keys,
