@@ -989,10 +989,9 @@ static rt_status render_impl(rt_ctx* c, const rt_camera* cams, uint32_t n_cams, 
     return fail(c, RT_ERR_ARG, "rt_render: trace_block must be a multiple of 32 up to 128");
   LaunchCfg lc;
   lc.block_trace = o.trace_block ? (int)o.trace_block : 128;
-  lc.block_shade = 256;
   lc.grid_trace = c->sms * (o.ctas_per_sm ? (int)o.ctas_per_sm : trace_blocks_per_sm(lc.block_trace));
   lc.grid_shadow = c->sms * (o.ctas_per_sm ? (int)o.ctas_per_sm : shadow_blocks_per_sm(lc.block_trace));
-  lc.grid_shade = c->sms * 8;
+  lc.sms = c->sms;
   lc.counting = c->counting;
   lc.record = o.probe_map_dev != nullptr;
   lc.variant = (int)o.trace_variant;
@@ -2003,10 +2002,9 @@ rt_status rt_render_photons(rt_ctx* c, const rt_camera* cams, uint32_t n_cams, u
   if (rt_status e = ensure_wave(c, cap)) return e;
   LaunchCfg lc;
   lc.block_trace = 128;
-  lc.block_shade = 256;
   lc.grid_trace = c->sms * trace_blocks_per_sm(lc.block_trace);
   lc.grid_shadow = c->sms * shadow_blocks_per_sm(lc.block_trace);
-  lc.grid_shade = c->sms * 8;
+  lc.sms = c->sms;
   lc.counting = false;
   lc.record = o.probe_map_dev != nullptr;
   lc.variant = 0;

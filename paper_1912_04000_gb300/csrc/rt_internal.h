@@ -263,7 +263,7 @@ constexpr int kDefaultShadowLeafBatch = 26;
 struct LaunchCfg {
   int grid_trace, block_trace;  // block_trace also sizes the sun-ray kernel's blocks
   int grid_shadow;
-  int grid_shade, block_shade;
+  int sms;  // SMs of the device
   bool counting;
   bool record;
   int variant;  // traversal: 0 = four-wide, leaf batching; binary: 1 = while-while, 2 = node-or-leaf steps,

@@ -1202,28 +1202,78 @@ __device__ __forceinline__ float photon_gather(const PhotonMaps& M, uint32_t map
   return sum;
 }
 
+// Appends of a block to N queues, one atomic per queue and turn of the whole
+// block: with one per warp, the half a million atomics of a wave on the same
+// two or three counters bounded the shading kernels (they are served one after
+// another, about one per nanosecond).  Two buffers, so that a warp
+// may enter its next turn while another reads this one's.
+template <int N>
+struct BlockAppend {
+  uint32_t first[2][N][8];  // per warp (at most 8): count, then first slot
+  // All threads of the block: the slots of the queues that this thread wants.
+  template <int M>
+  __device__ __forceinline__ void slots(uint32_t turn, const bool (&want)[M], uint32_t* const (&counter)[M],
+                                        uint32_t (&slot)[M]) {
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    uint32_t mask[N];
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      mask[q] = __ballot_sync(0xffffffffu, want[q]);
+      if (lane == 0) first[turn][q][warp] = (uint32_t)__popc(mask[q]);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < N; ++q)
+      if (warp == (uint32_t)q % nw) {
+        // lane w: warp w's count; exclusive sums over the (at most 8) warps
+        const uint32_t c = lane < nw ? first[turn][q][lane] : 0u;
+        uint32_t x = c;
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) {
+          const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+          if ((int)lane >= o) x += y;
+        }
+        uint32_t b = 0;
+        const uint32_t total = __shfl_sync(0xffffffffu, x, 7);
+        if (lane == 0 && total != 0u) b = atomicAdd(counter[q], total);
+        b = __shfl_sync(0xffffffffu, b, 0);
+        if (lane < nw) first[turn][q][lane] = b + x - c;
+      }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < N; ++q) slot[q] = first[turn][q][warp] + (uint32_t)__popc(mask[q] & ((1u << lane) - 1u));
+  }
+};
+
 // PM: photon-mapping camera pass -- at the first Lambertian vertex the path
 // adds (rho / pi) x the photon irradiance of both maps of pm and ends (its
 // sun ray, if any, finishes it).
-// three blocks of 256 per SM (<= 85 registers, no spills; unbounded, the
-// one-band shading took 102 registers and two blocks): measured 291 instead
-// of 304 ms per guided pass of the 2M-triangle nave, 375 instead of 377 ms
-// per render of the nave; four blocks (64 registers, spilled) were slower
-#ifndef SRT_SHADE_MIN_BLOCKS
-#define SRT_SHADE_MIN_BLOCKS 3
-#endif
+// Latency-bound: a chain of dependent reads (ray and hit, normal and radiance,
+// material row) per turn, so that resident warps count for more than the few
+// spilled registers they cost, and blocks are small so that their two
+// barriers per turn wait for few warps.  Two samples of the 1024 x 768 nave / one
+// of two guided 1024 x 768 views of the 2M-triangle nave (shading alone):
+// 3 blocks of 256 per SM, one atomic per warp and queue 47.2 / 29.2 ms; one per
+// block 37.2 / 24.6; as many blocks as are resident instead of 8 per SM
+// 34.8 / 23.1; 6 blocks of 128 31.8 / 21.1, 7 29.3 / 19.7, 8 28.7 / 19.4 (64
+// registers), 9 28.7 / 18.9, 10 29.8 / 20.0.  Four bands (512 x 384 crystal nave, 4
+// samples): 13.2 ms, then 11.5 with 3 blocks of 256, 10.3 with 4, 10.8 with 8 of 128.
+constexpr int kShadeThreads = 128, kShadeBlocksPerSm = 8;
+constexpr int kShade4Threads = 256, kShade4BlocksPerSm = 4;
 template <bool RECORD, bool GUIDED, bool PM = false>
-__global__ void __launch_bounds__(256, SRT_SHADE_MIN_BLOCKS) k_shade(DevScene S, DevSpectra P, WaveParams w, uint32_t k,
+__global__ void __launch_bounds__(kShadeThreads, kShadeBlocksPerSm) k_shade(DevScene S, DevSpectra P, WaveParams w, uint32_t k,
                                                const float4* __restrict__ qin, const float2* __restrict__ hit,
                                                float4* __restrict__ qout, float4* __restrict__ sq,
                                                float* __restrict__ Lbuf, uint32_t* __restrict__ sigbuf,
                                                Counters* cnt, uint32_t cap, double* __restrict__ accum,
                                                Probe probe, uint32_t* status, GuideWave gw, PhotonMaps pm) {
   const uint32_t count = min(cnt[k].q_count, cap);
-  const uint32_t lane = threadIdx.x & 31u;
   const uint32_t stride = gridDim.x * blockDim.x;
-  for (uint32_t base = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); base < count; base += stride) {
-    const uint32_t i = base + lane;
+  __shared__ BlockAppend<GUIDED ? 3 : 2> app;
+  uint32_t turn = 0;
+  // (every thread of the block makes the same number of turns)
+  for (uint32_t base = blockIdx.x * blockDim.x; base < count; base += stride, turn ^= 1u) {
+    const uint32_t i = base + threadIdx.x;
     bool emit_next = false, emit_shadow = false, emit_guide = false;
     float4 n0 = make_float4(0, 0, 0, 0), n1 = n0, s0 = n0, s1 = n0;
     float g_rho = 0.0f;
@@ -1385,10 +1435,13 @@ __global__ void __launch_bounds__(256, SRT_SHADE_MIN_BLOCKS) k_shade(DevScene S,
         if (RECORD) sigbuf[pid] = sg;
       }
     }
-    const uint32_t slot_n = warp_append(&cnt[k + 1].q_count, emit_next);
-    const uint32_t slot_s = warp_append(&cnt[k].s_count, emit_shadow);
+    const bool want[3] = {emit_next, emit_shadow, emit_guide};
+    uint32_t* const counter[3] = {&cnt[k + 1].q_count, &cnt[k].s_count, &cnt[k].g_count};
+    uint32_t slot[3];
+    app.slots(turn, want, counter, slot);
+    const uint32_t slot_n = slot[0], slot_s = slot[1];
     if (GUIDED) {
-      const uint32_t slot_g = warp_append(&cnt[k].g_count, emit_guide);
+      const uint32_t slot_g = slot[2];
       if (emit_guide) {
         if (slot_g < cap) {
           gw.gq[3 * slot_g] = n0;
@@ -1437,10 +1490,9 @@ __global__ void __launch_bounds__(256, SRT_SHADE_MIN_BLOCKS) k_shade(DevScene S,
 //     and the others stop (their radiance so far is kept).
 // "Carried" = throughput != 0; with one band left every rule is the
 // one-band rule of k_shade.  Each choice has the one-band expectation per
-// band, so the four-band estimate of every band is unbiased.  Three blocks
-// of 256 per SM (80 registers, a few bytes spilled) beat two blocks at 92.
+// band, so the four-band estimate of every band is unbiased.
 template <bool RECORD>
-__global__ void __launch_bounds__(256, 3) k_shade4(DevScene S, DevSpectra P, WaveParams w, uint32_t k,
+__global__ void __launch_bounds__(kShade4Threads, kShade4BlocksPerSm) k_shade4(DevScene S, DevSpectra P, WaveParams w, uint32_t k,
                                                 const float4* __restrict__ qin, const float2* __restrict__ hit,
                                                 float4* __restrict__ qout, float4* __restrict__ sq,
                                                 float4* __restrict__ L4, float4* __restrict__ T4,
@@ -1448,10 +1500,11 @@ __global__ void __launch_bounds__(256, 3) k_shade4(DevScene S, DevSpectra P, Wav
                                                 Counters* cnt, uint32_t cap, double* __restrict__ accum,
                                                 Probe probe, uint32_t* status) {
   const uint32_t count = min(cnt[k].q_count, cap);
-  const uint32_t lane = threadIdx.x & 31u;
   const uint32_t stride = gridDim.x * blockDim.x;
-  for (uint32_t base = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); base < count; base += stride) {
-    const uint32_t i = base + lane;
+  __shared__ BlockAppend<2> app;
+  uint32_t turn = 0;
+  for (uint32_t base = blockIdx.x * blockDim.x; base < count; base += stride, turn ^= 1u) {
+    const uint32_t i = base + threadIdx.x;
     bool emit_next = false, emit_shadow = false;
     float4 n0 = make_float4(0, 0, 0, 0), n1 = n0, s0 = n0, s1 = n0;
     if (i < count) {
@@ -1684,8 +1737,11 @@ __global__ void __launch_bounds__(256, 3) k_shade4(DevScene S, DevSpectra P, Wav
       }
       if (emit_next) T4[pid] = make_float4(T[0], T[1], T[2], T[3]);
     }
-    const uint32_t slot_n = warp_append(&cnt[k + 1].q_count, emit_next);
-    const uint32_t slot_s = warp_append(&cnt[k].s_count, emit_shadow);
+    const bool want[2] = {emit_next, emit_shadow};
+    uint32_t* const counter[2] = {&cnt[k + 1].q_count, &cnt[k].s_count};
+    uint32_t slot[2];
+    app.slots(turn, want, counter, slot);
+    const uint32_t slot_n = slot[0], slot_s = slot[1];
     if (emit_next) {
       if (slot_n < cap) {
         __stcs(qout + 2 * slot_n, n0);
@@ -2328,7 +2384,10 @@ void launch_wave(const LaunchCfg& lcfg, const DevScene& S, const DevSpectra& P, 
   auto blocks = [&](int block) { return (int)((w.n + (uint32_t)block - 1u) / (uint32_t)block); };
   lc.grid_trace = std::min(lc.grid_trace, blocks(lc.block_trace));
   lc.grid_shadow = std::min(lc.grid_shadow, blocks(lc.block_trace));
-  lc.grid_shade = std::min(lc.grid_shade, blocks(lc.block_shade));
+  // shading: as many blocks as are resident at once, each with the same share
+  const int block_shade = w.nb == 4u ? kShade4Threads : kShadeThreads;
+  const int grid_shade =
+      std::min(lc.sms * (w.nb == 4u ? kShade4BlocksPerSm : kShadeBlocksPerSm), blocks(block_shade));
   const bool rec = lc.record;
   if (tm) tm->begin(STG_CAMERA, st);
   k_camera<<<grid_for(w.n, 256), 256, 0, st>>>(cams, n_cams, w, b.q[1], b.L, b.sig, b.cnt, rec, b.L4, b.T4, b.cap,
@@ -2350,31 +2409,31 @@ void launch_wave(const LaunchCfg& lcfg, const DevScene& S, const DevSpectra& P, 
     if (tm) tm->begin(STG_SHADE, st);
     if (w.nb == 4u) {
       if (rec)
-        k_shade4<true><<<lc.grid_shade, lc.block_shade, 0, st>>>(S, P, w, k, qin, b.hit, qout, b.sq, b.L4, b.T4, b.C4,
+        k_shade4<true><<<grid_shade, block_shade, 0, st>>>(S, P, w, k, qin, b.hit, qout, b.sq, b.L4, b.T4, b.C4,
                                                                  b.sig, b.cnt, b.cap, accum, probe, b.status);
       else
-        k_shade4<false><<<lc.grid_shade, lc.block_shade, 0, st>>>(S, P, w, k, qin, b.hit, qout, b.sq, b.L4, b.T4,
+        k_shade4<false><<<grid_shade, block_shade, 0, st>>>(S, P, w, k, qin, b.hit, qout, b.sq, b.L4, b.T4,
                                                                   b.C4, b.sig, b.cnt, b.cap, accum, probe, b.status);
     } else if (pm) {
       if (rec)
-        k_shade<true, false, true><<<lc.grid_shade, lc.block_shade, 0, st>>>(
+        k_shade<true, false, true><<<grid_shade, block_shade, 0, st>>>(
             S, P, w, k, qin, b.hit, qout, b.sq, b.L, b.sig, b.cnt, b.cap, accum, probe, b.status, gw, *pm);
       else
-        k_shade<false, false, true><<<lc.grid_shade, lc.block_shade, 0, st>>>(
+        k_shade<false, false, true><<<grid_shade, block_shade, 0, st>>>(
             S, P, w, k, qin, b.hit, qout, b.sq, b.L, b.sig, b.cnt, b.cap, accum, probe, b.status, gw, *pm);
     } else if (guided) {
       if (rec)
-        k_shade<true, true><<<lc.grid_shade, lc.block_shade, 0, st>>>(S, P, w, k, qin, b.hit, qout, b.sq, b.L, b.sig,
+        k_shade<true, true><<<grid_shade, block_shade, 0, st>>>(S, P, w, k, qin, b.hit, qout, b.sq, b.L, b.sig,
                                                                      b.cnt, b.cap, accum, probe, b.status, gw, PhotonMaps{});
       else
-        k_shade<false, true><<<lc.grid_shade, lc.block_shade, 0, st>>>(S, P, w, k, qin, b.hit, qout, b.sq, b.L, b.sig,
+        k_shade<false, true><<<grid_shade, block_shade, 0, st>>>(S, P, w, k, qin, b.hit, qout, b.sq, b.L, b.sig,
                                                                       b.cnt, b.cap, accum, probe, b.status, gw, PhotonMaps{});
     } else {
       if (rec)
-        k_shade<true, false><<<lc.grid_shade, lc.block_shade, 0, st>>>(S, P, w, k, qin, b.hit, qout, b.sq, b.L, b.sig,
+        k_shade<true, false><<<grid_shade, block_shade, 0, st>>>(S, P, w, k, qin, b.hit, qout, b.sq, b.L, b.sig,
                                                                       b.cnt, b.cap, accum, probe, b.status, gw, PhotonMaps{});
       else
-        k_shade<false, false><<<lc.grid_shade, lc.block_shade, 0, st>>>(S, P, w, k, qin, b.hit, qout, b.sq, b.L,
+        k_shade<false, false><<<grid_shade, block_shade, 0, st>>>(S, P, w, k, qin, b.hit, qout, b.sq, b.L,
                                                                        b.sig, b.cnt, b.cap, accum, probe, b.status, gw, PhotonMaps{});
     }
     if (tm) tm->end(STG_SHADE, st);

@@ -136,10 +136,9 @@ extern "C" rt_status rt_render_static(rt_ctx* c, const rt_camera* cams, uint32_t
   STATIC_TRY(cudaMemsetAsync(b.tot, 0, sizeof(Totals), st));
   LaunchCfg lc;
   lc.block_trace = 128;
-  lc.block_shade = 256;
   lc.grid_trace = v.sms * trace_blocks_per_sm(lc.block_trace);
   lc.grid_shadow = v.sms * shadow_blocks_per_sm(lc.block_trace);
-  lc.grid_shade = v.sms * 8;
+  lc.sms = v.sms;
   lc.counting = false;
   lc.record = false;
   lc.variant = 0;
