@@ -63,7 +63,8 @@ typedef enum {
 } rt_material_type;
 
 typedef enum {
-  RT_XYZ_BF16X3 = 0, /* tensor cores, BF16 operands split in three terms, FP32 accumulate */
+  RT_XYZ_BF16X3 = 0, /* FP32 accuracy: what three BF16 terms per operand carry, computed in FP32;
+                        at most 192 bands */
   RT_XYZ_BF16 = 1,   /* tensor cores, plain BF16 operands, FP32 accumulate */
   RT_XYZ_FP64 = 2    /* CUDA cores, FP64 (reference mode) */
 } rt_xyz_mode;

@@ -170,13 +170,4 @@ __device__ __forceinline__ uint32_t tc_bf16x2_bits(float lo, float hi) {
   return r;
 }
 
-// v = hi + mid + lo with each term the BF16 rounding of the remainder.
-__device__ __forceinline__ void tc_split3(float v, uint16_t& h, uint16_t& m, uint16_t& l) {
-  h = tc_bf16_bits(v);
-  const float r1 = v - tc_bf16_val(h);
-  m = tc_bf16_bits(r1);
-  const float r2 = r1 - tc_bf16_val(m);
-  l = tc_bf16_bits(r2);
-}
-
 }  // namespace srt

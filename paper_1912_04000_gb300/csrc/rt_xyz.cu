@@ -2,19 +2,18 @@
 //
 //   xyz[p][c] = sum_j (spectral[p][j] / spp) * w[j][c]
 //
-// RT_XYZ_BF16X3 / RT_XYZ_BF16: 5th-generation tensor cores (tcgen05.mma,
-// accumulator in tensor memory).  One CTA (128 threads) processes tiles of
-// 128 pixels: the FP64 rows are streamed from HBM with coalesced 16-byte
-// loads, rounded to FP32 (integer operations on the IEEE fields), scaled by
-// 1/spp and split into BF16 terms v = hi + mid + lo (each the BF16 rounding of
-// the remainder), written to shared memory in the K-major, non-swizzled
-// canonical layout (8 x 16-byte core matrices).
-// One thread issues D[128 x 16] += A[128 x 16] B[16 x 16]
-// for every 16-band slice: with the three-term split of both operands the six
-// products hi.hi, hi.mid, mid.hi, hi.lo, lo.hi, mid.mid carry FP32-level
-// accuracy (the dropped terms are below 2^-26 relative, after Henry, Tang and
-// Heinecke, ARITH 2019); RT_XYZ_BF16 uses hi.hi only.  The FP32 accumulator is
-// read back with tcgen05.ld (warp w owns TMEM lanes 32w..32w+31 = pixels).
+// RT_XYZ_BF16X3 (the default, FP32-level accuracy): k_xyz_f32, FP32 FMAs on
+// the CUDA cores.  Three columns make 6 flops per 8 bytes read: the path is
+// bound by HBM, and an operand must reach a tensor core through shared memory
+// as three BF16 terms, which cost more than the FMAs they replace.
+//
+// RT_XYZ_BF16: 5th-generation tensor cores (tcgen05.mma, accumulator in tensor
+// memory).  A CTA processes tiles of 128 pixels: the FP64 rows are rounded to
+// FP32 (integer operations on the IEEE fields), scaled by 1/spp and rounded to
+// BF16, written to shared memory in the K-major, non-swizzled canonical layout
+// (8 x 16-byte core matrices).  One thread issues D[128 x 16] += A[128 x 16]
+// B[16 x 16] for every 16-band slice.  The FP32 accumulator is read back with
+// tcgen05.ld (warp w owns TMEM lanes 32w..32w+31 = pixels).
 //
 // RT_XYZ_FP64: CUDA cores, FP64, the reference mode.
 #include <cstdint>
@@ -87,15 +86,17 @@ __device__ __forceinline__ float f64_to_f32_rz(uint32_t lo, uint32_t hi) {
   return __uint_as_float(((hi >> 20) & 0x7FFu) > 896u ? (bits | sign) : sign);
 }
 
-// v = hi + mid + lo exactly, each term a BF16 value: hi keeps the top 8
-// significant bits of v (truncation), mid the top 8 of the remainder, lo the
-// rest (at most 8 bits, exact).  Returned as the BF16 bit patterns in the
-// upper halves of three words.
-__device__ __forceinline__ void split3_trunc(float v, uint32_t& h, uint32_t& m, uint32_t& l) {
-  h = __float_as_uint(v) & 0xFFFF0000u;
-  const float r1 = v - __uint_as_float(h);
-  m = __float_as_uint(r1) & 0xFFFF0000u;
-  l = __float_as_uint(r1 - __uint_as_float(m));
+// FP64 -> FP32, nearest (ties away from zero): one bit more than the 23 kept,
+// plus one, halved.  Magnitudes below the FP32 normal range give signed zero.
+// top keeps the largest rebiased high word: past kTopF32 a value lies above
+// the FP32 range or is not finite, and its result is wrong.
+constexpr int kTopF32 = (1150 - 896) << 20;
+__device__ __forceinline__ float f64_to_f32_rn(uint2 d, int& top) {
+  const int t = (int)((d.y & 0x7FFFFFFFu) - (896u << 20));
+  top = max(top, t);
+  const uint32_t bits = (__funnelshift_l(d.x, (uint32_t)t, 4) + 1u) >> 1;
+  const uint32_t sign = d.y & 0x80000000u;
+  return __uint_as_float(t >= (1 << 20) ? (bits | sign) : sign);
 }
 
 constexpr int kTileM = 128;        // pixels per tile = MMA M = TMEM lanes
@@ -112,26 +113,20 @@ constexpr int kUnroll = 8;
 // index of a tile (e < 128 * 192).
 __global__ void __launch_bounds__(kXyzThreads) k_xyz_tc(const double* __restrict__ s, uint64_t np, uint32_t bc,
                                                         uint32_t nk, uint32_t inv_bc, const float* __restrict__ w,
-                                                        double inv_spp, float* __restrict__ xyz, int n_split,
-                                                        uint32_t* status) {
+                                                        double inv_spp, float* __restrict__ xyz, uint32_t* status) {
   extern __shared__ __align__(1024) unsigned char smem[];
-  unsigned char* A = smem;                                   // [3][nk][4096]
-  unsigned char* Bm = smem + 3u * nk * kATile;               // [3][nk][512]
-  uint64_t* mbar = (uint64_t*)(Bm + 3u * nk * kBTile);
+  unsigned char* A = smem;                                   // [nk][4096]
+  unsigned char* Bm = smem + nk * kATile;                    // [nk][512]
+  uint64_t* mbar = (uint64_t*)(Bm + nk * kBTile);
   uint32_t* tslot = (uint32_t*)(mbar + 1);
   const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31u;
 
-  // zero A (its padded K columns stay zero) and build the split weights
-  for (uint32_t i = tid; i < 3u * nk * kATile / 16u; i += blockDim.x) ((uint4*)A)[i] = make_uint4(0, 0, 0, 0);
+  // zero A (its padded K columns stay zero) and build the weight tile
+  for (uint32_t i = tid; i < nk * kATile / 16u; i += blockDim.x) ((uint4*)A)[i] = make_uint4(0, 0, 0, 0);
   for (uint32_t i = tid; i < (uint32_t)kMmaN * nk * 16u; i += blockDim.x) {
     const uint32_t n = i / (nk * 16u), k = i - n * nk * 16u;
     const float v = (n < 3u && k < bc) ? w[3u * k + n] : 0.0f;
-    uint16_t h, m, l;
-    tc_split3(v, h, m, l);
-    const uint32_t off = (k >> 4) * kBTile + tc_kmajor_off(n, k & 15u);
-    *(uint16_t*)(Bm + off) = h;
-    *(uint16_t*)(Bm + nk * kBTile + off) = m;
-    *(uint16_t*)(Bm + 2u * nk * kBTile + off) = l;
+    *(uint16_t*)(Bm + (k >> 4) * kBTile + tc_kmajor_off(n, k & 15u)) = tc_bf16_bits(v);
   }
   if (tid == 0) {
     tc_mbar_init(mbar, 1);
@@ -143,8 +138,6 @@ __global__ void __launch_bounds__(kXyzThreads) k_xyz_tc(const double* __restrict
   tc_fence_after();
   const uint32_t tmem = *tslot;
 
-  // products (a split, b split)
-  const uint32_t pa[6] = {0, 0, 1, 0, 2, 1}, pb[6] = {0, 1, 0, 2, 0, 1};
   const uint64_t ntiles = (np + kTileM - 1) / kTileM;
   const float inv_spp_f = (float)inv_spp;
   uint32_t phase = 0;
@@ -179,14 +172,7 @@ __global__ void __launch_bounds__(kXyzThreads) k_xyz_tc(const double* __restrict
           if (ee < nel) {
             const uint32_t r = __umulhi(ee, inv_bc), k = ee - r * bc;
             const float val = f64_to_f32<true>(h2 ? v[u].y : v[u].x) * inv_spp_f;
-            uint16_t hh, mm, ll;
-            tc_split3(val, hh, mm, ll);
-            const uint32_t off = (k >> 4) * kATile + tc_kmajor_off(r, k & 15u);
-            *(uint16_t*)(A + off) = hh;
-            if (n_split > 1) {
-              *(uint16_t*)(A + nk * kATile + off) = mm;
-              *(uint16_t*)(A + 2u * nk * kATile + off) = ll;
-            }
+            *(uint16_t*)(A + (k >> 4) * kATile + tc_kmajor_off(r, k & 15u)) = tc_bf16_bits(val);
           }
         }
       }
@@ -195,15 +181,9 @@ __global__ void __launch_bounds__(kXyzThreads) k_xyz_tc(const double* __restrict
     __syncthreads();
     if (tid == 0) {
       tc_fence_after();
-      const int nprod = n_split > 1 ? 6 : 1;
-      uint32_t acc = 0;
       for (uint32_t kb = 0; kb < nk; ++kb)
-        for (int pr = 0; pr < nprod; ++pr) {
-          const uint64_t da = tc_smem_desc(smem_u32(A + pa[pr] * nk * kATile + kb * kATile));
-          const uint64_t db = tc_smem_desc(smem_u32(Bm + pb[pr] * nk * kBTile + kb * kBTile));
-          tc_mma_bf16(tmem, da, db, kIdesc, acc);
-          acc = 1;
-        }
+        tc_mma_bf16(tmem, tc_smem_desc(smem_u32(A + kb * kATile)), tc_smem_desc(smem_u32(Bm + kb * kBTile)), kIdesc,
+                    kb > 0 ? 1u : 0u);
       tc_commit(mbar);
     }
     const int timed_out = __syncthreads_or(tc_mbar_wait(mbar, phase, 1u << 24) ? 0 : 1);
@@ -232,11 +212,11 @@ __global__ void __launch_bounds__(kXyzThreads) k_xyz_tc(const double* __restrict
 }
 
 // ---------------------------------------------------------------------------
-// TMA-pipelined variant (the default when it fits in shared memory): a tile of
+// TMA-pipelined variant (RT_XYZ_BF16 where it fits in shared memory): a tile of
 // 128 pixels arrives as two halves of 64 rows, each one bulk copy (the rows
 // are contiguous) into its own shared buffer, completion counted on an
-// mbarrier.  Each half is converted (divide by spp, FP32, three-term BF16
-// split, 16-byte stores of 8 K-consecutive values into the canonical layout)
+// mbarrier.  Each half is converted (FP32, divide by spp, BF16, 16-byte stores
+// of 8 K-consecutive values into the canonical layout)
 // as soon as it lands, and the copy of the same half of the CTA's next tile is
 // issued as soon as the buffer is read, so HBM traffic overlaps conversion,
 // MMA and epilogue.  A tail tile whose halves are not full is read with
@@ -252,25 +232,20 @@ constexpr int kXyzTmaThreads = 512;
 
 __global__ void __launch_bounds__(kXyzTmaThreads, 1) k_xyz_tma(const double* __restrict__ s, uint64_t np, uint32_t bc,
                                                             uint32_t nk, const float* __restrict__ w, double inv_spp,
-                                                            float* __restrict__ xyz, int n_split, uint32_t* status) {
+                                                            float* __restrict__ xyz, uint32_t* status) {
   extern __shared__ __align__(1024) unsigned char smem[];
   const uint32_t half_bytes = kHalf * bc * 8u;  // a multiple of 512
   unsigned char* raw0 = smem;
   unsigned char* A = smem + 2u * half_bytes;
-  unsigned char* Bm = A + 3u * nk * kATile;
-  uint64_t* mb = (uint64_t*)(Bm + 3u * nk * kBTile);  // [0], [1]: raw halves, [2]: MMA
+  unsigned char* Bm = A + nk * kATile;
+  uint64_t* mb = (uint64_t*)(Bm + nk * kBTile);  // [0], [1]: raw halves, [2]: MMA
   uint32_t* tslot = (uint32_t*)(mb + 3);
   const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31u;
-  for (uint32_t i = tid; i < 3u * nk * kATile / 16u; i += blockDim.x) ((uint4*)A)[i] = make_uint4(0, 0, 0, 0);
+  for (uint32_t i = tid; i < nk * kATile / 16u; i += blockDim.x) ((uint4*)A)[i] = make_uint4(0, 0, 0, 0);
   for (uint32_t i = tid; i < (uint32_t)kMmaN * nk * 16u; i += blockDim.x) {
     const uint32_t n = i / (nk * 16u), k = i - n * nk * 16u;
     const float v = (n < 3u && k < bc) ? w[3u * k + n] : 0.0f;
-    uint16_t h, m, l;
-    tc_split3(v, h, m, l);
-    const uint32_t off = (k >> 4) * kBTile + tc_kmajor_off(n, k & 15u);
-    *(uint16_t*)(Bm + off) = h;
-    *(uint16_t*)(Bm + nk * kBTile + off) = m;
-    *(uint16_t*)(Bm + 2u * nk * kBTile + off) = l;
+    *(uint16_t*)(Bm + (k >> 4) * kBTile + tc_kmajor_off(n, k & 15u)) = tc_bf16_bits(v);
   }
   if (tid == 0) {
     for (int i = 0; i < 3; ++i) tc_mbar_init(mb + i, 1);
@@ -296,7 +271,6 @@ __global__ void __launch_bounds__(kXyzTmaThreads, 1) k_xyz_tma(const double* __r
         inflight[h] = true;
         if (tid == 0) issue(blockIdx.x, h);
       }
-  const uint32_t pa[6] = {0, 0, 1, 0, 2, 1}, pb[6] = {0, 1, 0, 2, 0, 1};
   uint32_t ph[2] = {0u, 0u}, phm = 0u;
   bool ok = true;
   for (uint64_t tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
@@ -323,50 +297,19 @@ __global__ void __launch_bounds__(kXyzTmaThreads, 1) k_xyz_tma(const double* __r
       const uint32_t items = kHalf * 2u * nk;
       for (uint32_t it = tid; it < items; it += blockDim.x) {
         const uint32_t r = it % kHalf, g8 = it / kHalf;
-        uint32_t hb[8], mb_[8], lb[8];
+        float v[8];
         const double* rowp = (const double*)raw + r * bc + 8u * g8;
-        if (r < rh && 8u * g8 + 8u <= bc) {
-          // full group: no bounds checks
 #pragma unroll
-          for (int e = 0; e < 8; ++e) {
+        for (int e = 0; e < 8; ++e) {
+          v[e] = 0.0f;
+          if (r < rh && 8u * g8 + (uint32_t)e < bc) {
             const uint2 wv = *(const uint2*)(rowp + e);
-            const float v = f64_to_f32_rz(wv.x, wv.y) * inv_spp_f;
-            if (n_split > 1) {
-              split3_trunc(v, hb[e], mb_[e], lb[e]);
-            } else {
-              const uint32_t u = __float_as_uint(v);
-              hb[e] = (u + 0x7FFFu + ((u >> 16) & 1u)) & 0xFFFF0000u;  // BF16, round to nearest even
-            }
-          }
-        } else {
-#pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            const uint32_t j = 8u * g8 + (uint32_t)e;
-            float v = 0.0f;
-            if (r < rh && j < bc) {
-              const uint2 wv = *(const uint2*)(rowp + e);
-              v = f64_to_f32_rz(wv.x, wv.y) * inv_spp_f;
-            }
-            if (n_split > 1) {
-              split3_trunc(v, hb[e], mb_[e], lb[e]);
-            } else {
-              const uint32_t u = __float_as_uint(v);
-              hb[e] = (u + 0x7FFFu + ((u >> 16) & 1u)) & 0xFFFF0000u;
-            }
+            v[e] = f64_to_f32_rz(wv.x, wv.y) * inv_spp_f;
           }
         }
-        // pairs of upper halves into words, the first value in the low half
-        const uint32_t off = (g8 >> 1) * kATile + tc_kmajor_off(h * kHalf + r, (g8 & 1u) * 8u);
-        *(uint4*)(A + off) = make_uint4(__byte_perm(hb[0], hb[1], 0x7632), __byte_perm(hb[2], hb[3], 0x7632),
-                                        __byte_perm(hb[4], hb[5], 0x7632), __byte_perm(hb[6], hb[7], 0x7632));
-        if (n_split > 1) {
-          *(uint4*)(A + nk * kATile + off) =
-              make_uint4(__byte_perm(mb_[0], mb_[1], 0x7632), __byte_perm(mb_[2], mb_[3], 0x7632),
-                         __byte_perm(mb_[4], mb_[5], 0x7632), __byte_perm(mb_[6], mb_[7], 0x7632));
-          *(uint4*)(A + 2u * nk * kATile + off) =
-              make_uint4(__byte_perm(lb[0], lb[1], 0x7632), __byte_perm(lb[2], lb[3], 0x7632),
-                         __byte_perm(lb[4], lb[5], 0x7632), __byte_perm(lb[6], lb[7], 0x7632));
-        }
+        *(uint4*)(A + (g8 >> 1) * kATile + tc_kmajor_off(h * kHalf + r, (g8 & 1u) * 8u)) =
+            make_uint4(tc_bf16x2_bits(v[0], v[1]), tc_bf16x2_bits(v[2], v[3]), tc_bf16x2_bits(v[4], v[5]),
+                       tc_bf16x2_bits(v[6], v[7]));
       }
       // the buffer is read: refill it with the same half of the next tile
       __syncthreads();
@@ -384,15 +327,9 @@ __global__ void __launch_bounds__(kXyzTmaThreads, 1) k_xyz_tma(const double* __r
     __syncthreads();
     if (tid == 0) {
       tc_fence_after();
-      const int nprod = n_split > 1 ? 6 : 1;
-      uint32_t acc = 0;
       for (uint32_t kb = 0; kb < nk; ++kb)
-        for (int pr = 0; pr < nprod; ++pr) {
-          const uint64_t da = tc_smem_desc(smem_u32(A + pa[pr] * nk * kATile + kb * kATile));
-          const uint64_t db = tc_smem_desc(smem_u32(Bm + pb[pr] * nk * kBTile + kb * kBTile));
-          tc_mma_bf16(tmem, da, db, kIdesc, acc);
-          acc = 1;
-        }
+        tc_mma_bf16(tmem, tc_smem_desc(smem_u32(A + kb * kATile)), tc_smem_desc(smem_u32(Bm + kb * kBTile)), kIdesc,
+                    kb > 0 ? 1u : 0u);
       tc_commit(mb + 2);
     }
     const int timed_out = __syncthreads_or(tc_mbar_wait(mb + 2, phm, 1u << 24) ? 0 : 1);
@@ -426,14 +363,145 @@ __global__ void __launch_bounds__(kXyzTmaThreads, 1) k_xyz_tma(const double* __r
 
 size_t xyz_tma_smem(uint32_t band_count) {
   const uint32_t nk = (band_count + 15) / 16;
-  return 2ull * kHalf * band_count * 8ull + 3ull * nk * kATile + 3ull * nk * kBTile + 64;
+  return 2ull * kHalf * band_count * 8ull + (size_t)nk * kATile + (size_t)nk * kBTile + 64;
+}
+
+// ---------------------------------------------------------------------------
+// FP32 contraction (RT_XYZ_BF16X3).  Bound by HBM: 8 bytes per (pixel, band)
+// for some 15 instructions.  A stage is 32 RPT pixels, whose rows are
+// contiguous: one bulk copy (TMA) into shared memory, the CTA's next ones in
+// flight meanwhile.  Eight lanes share RPT pixels, lane l their bands l, l + 8,
+// ... (a row-per-lane order would meet in the same banks for even band
+// counts), and add up over the eight.  The last, short stage is read from
+// global memory.  786,432 pixels x 81 bands: 195 us with BF16 triples on
+// tensor cores (one CTA per SM; conversion, MMAs and epilogue of a tile in
+// turn), 198 us here with a pixel per eight lanes and a branch per conversion,
+// 103 us with two (the kernel alone 79 us, 6.4 TB/s).
+// ---------------------------------------------------------------------------
+constexpr int kF32Threads = 256;
+constexpr uint32_t kF32Stages = 4;
+constexpr uint32_t kF32Smem = 110u * 1024u;  // two CTAs per SM
+
+// pixels per eight lanes: two while two stages of 64 pixels fit
+uint32_t xyz_f32_rpt(uint32_t bc) { return 2u * 64u * bc * 8u + 16u * bc + 64u <= kF32Smem ? 2u : 1u; }
+uint32_t xyz_f32_stages(uint32_t bc) {
+  const uint32_t fit = (kF32Smem - 16u * bc - 64u) / (32u * xyz_f32_rpt(bc) * bc * 8u);
+  return fit > kF32Stages ? kF32Stages : fit;
+}
+size_t xyz_f32_smem(uint32_t bc) {
+  return (size_t)xyz_f32_stages(bc) * 32u * xyz_f32_rpt(bc) * bc * 8u + 16u * bc + 64u;
+}
+
+template <int RPT>
+__global__ void __launch_bounds__(kF32Threads, 2)
+    k_xyz_f32(const double* __restrict__ s, uint64_t np, uint32_t bc, uint32_t n_stages, const float* __restrict__ w,
+              float inv_spp, float* __restrict__ xyz, uint32_t* status) {
+  extern __shared__ __align__(1024) unsigned char smem[];
+  constexpr uint32_t kRows = 32u * RPT;
+  const uint32_t stage_bytes = kRows * bc * 8u;  // a multiple of 256
+  float4* W = (float4*)(smem + n_stages * stage_bytes);
+  uint64_t* full = (uint64_t*)(W + bc);
+  const uint32_t tid = threadIdx.x, row = tid >> 3, l = tid & 7u;
+  for (uint32_t j = tid; j < bc; j += blockDim.x) W[j] = make_float4(w[3u * j], w[3u * j + 1], w[3u * j + 2], 0.0f);
+  if (tid == 0) {
+    for (uint32_t i = 0; i < n_stages; ++i) tc_mbar_init(full + i, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  const uint64_t nt = (np + kRows - 1) / kRows;
+  auto whole = [&](uint64_t t) { return (t + 1) * kRows <= np; };
+  auto issue = [&](uint64_t t, uint32_t st) {
+    tc_mbar_expect_tx(full + st, stage_bytes);
+    tc_bulk_g2s(smem + st * stage_bytes, s + t * kRows * bc, stage_bytes, full + st);
+  };
+  if (tid == 0)
+    for (uint32_t i = 0; i < n_stages; ++i) {
+      const uint64_t t = blockIdx.x + (uint64_t)i * gridDim.x;
+      if (t < nt && whole(t)) issue(t, i);
+    }
+  uint32_t st = 0, phase = 0;
+  for (uint64_t t = blockIdx.x; t < nt; t += gridDim.x) {
+    const bool staged = whole(t);
+    if (staged && __syncthreads_or(tc_mbar_wait(full + st, phase, 1u << 24) ? 0 : 1)) {
+      if (tid == 0) {
+        atomicOr(status, ST_ITER);
+        // copies still in flight write this CTA's memory: wait (bounded) for them
+        for (uint32_t i = 1; i < n_stages; ++i) {
+          const uint64_t u = t + (uint64_t)i * gridDim.x;
+          const uint32_t si = st + i < n_stages ? st + i : st + i - n_stages;
+          if (u < nt && whole(u)) tc_mbar_wait(full + si, si < st ? phase ^ 1u : phase, 1u << 24);
+        }
+      }
+      return;
+    }
+    // the eight lanes' pixels: rows row, row + 32 of the stage
+    const uint64_t p0 = t * kRows + row;
+    const uint2* v[RPT];
+    float x[RPT], y[RPT], z[RPT];
+    int top = 0;
+#pragma unroll
+    for (int q = 0; q < RPT; ++q) {
+      // (past the image's end: its last pixel, whose result is not stored)
+      const uint64_t p = min(p0 + 32u * (uint32_t)q, np - 1);
+      v[q] = staged ? (const uint2*)(smem + st * stage_bytes) + (row + 32u * (uint32_t)q) * bc
+                    : (const uint2*)(s + p * bc);
+      x[q] = y[q] = z[q] = 0.0f;
+    }
+#pragma unroll 4
+    for (uint32_t j = l; j < bc; j += 8u) {
+      const float4 c = W[j];
+#pragma unroll
+      for (int q = 0; q < RPT; ++q) {
+        const float f = f64_to_f32_rn(v[q][j], top);
+        x[q] = fmaf(f, c.x, x[q]);
+        y[q] = fmaf(f, c.y, y[q]);
+        z[q] = fmaf(f, c.z, z[q]);
+      }
+    }
+    if (top > kTopF32) {  // a sum above the FP32 range, an infinity or a NaN: by the conversion instruction
+#pragma unroll
+      for (int q = 0; q < RPT; ++q) {
+        x[q] = y[q] = z[q] = 0.0f;
+        for (uint32_t j = l; j < bc; j += 8u) {
+          const float4 c = W[j];
+          const uint2 d = v[q][j];
+          const float f = (float)__hiloint2double((int)d.y, (int)d.x);
+          x[q] = fmaf(f, c.x, x[q]);
+          y[q] = fmaf(f, c.y, y[q]);
+          z[q] = fmaf(f, c.z, z[q]);
+        }
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < RPT; ++q) {
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) {
+        x[q] += __shfl_xor_sync(0xffffffffu, x[q], o);
+        y[q] += __shfl_xor_sync(0xffffffffu, y[q], o);
+        z[q] += __shfl_xor_sync(0xffffffffu, z[q], o);
+      }
+      const uint64_t p = p0 + 32u * (uint32_t)q;
+      if (p < np && l < 3u) xyz[3 * p + l] = (l == 0 ? x[q] : (l == 1 ? y[q] : z[q])) * inv_spp;
+    }
+    // the stage is read: refill it
+    __syncthreads();
+    const uint64_t next = t + (uint64_t)n_stages * gridDim.x;
+    if (tid == 0 && staged && next < nt && whole(next)) {
+      tc_fence_async_smem();
+      issue(next, st);
+    }
+    if (++st == n_stages) {
+      st = 0;
+      phase ^= 1u;
+    }
+  }
 }
 
 }  // namespace
 
 size_t xyz_tc_smem(uint32_t band_count) {
   const uint32_t nk = (band_count + 15) / 16;
-  return 3ull * nk * kATile + 3ull * nk * kBTile + 16;
+  return (size_t)nk * kATile + (size_t)nk * kBTile + 16;
 }
 
 void launch_xyz(const double* spectral, uint64_t n_pixels, const XyzWeights& w, uint32_t spp, int mode, float* xyz,
@@ -447,6 +515,17 @@ void launch_xyz(const double* spectral, uint64_t n_pixels, const XyzWeights& w, 
     k_xyz_fp64<<<(unsigned)grid, block, smem, st>>>(spectral, n_pixels, w.band_count, w.w32, 1.0 / (double)spp, xyz);
     return;
   }
+  if (mode == 0) {
+    const size_t smem = xyz_f32_smem(w.band_count);
+    const uint32_t rpt = xyz_f32_rpt(w.band_count), n_stages = xyz_f32_stages(w.band_count);
+    auto* kernel = rpt == 2 ? k_xyz_f32<2> : k_xyz_f32<1>;
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const uint64_t nt = (n_pixels + 32 * rpt - 1) / (32 * rpt);
+    const unsigned grid = (unsigned)(nt < 2ull * (uint64_t)sms ? nt : 2ull * (uint64_t)sms);
+    kernel<<<grid, kF32Threads, smem, st>>>(spectral, n_pixels, w.band_count, n_stages, w.w32, (float)(1.0 / (double)spp),
+                                          xyz, status);
+    return;
+  }
   const uint32_t nk = (w.band_count + 15) / 16;
   const size_t tsmem = xyz_tma_smem(w.band_count);
   if (tsmem <= 227u * 1024u && ((uintptr_t)spectral & 15u) == 0) {
@@ -455,7 +534,7 @@ void launch_xyz(const double* spectral, uint64_t n_pixels, const XyzWeights& w, 
     uint64_t grid = (uint64_t)sms;
     if (grid > ntiles) grid = ntiles;
     k_xyz_tma<<<(unsigned)grid, kXyzTmaThreads, tsmem, st>>>(spectral, n_pixels, w.band_count, nk, w.w32,
-                                                         1.0 / (double)spp, xyz, mode == 0 ? 3 : 1, status);
+                                                         1.0 / (double)spp, xyz, status);
     return;
   }
   const size_t smem = xyz_tc_smem(w.band_count);
@@ -468,7 +547,7 @@ void launch_xyz(const double* spectral, uint64_t n_pixels, const XyzWeights& w, 
   if (grid > ntiles) grid = ntiles;
   const uint32_t inv_bc = (uint32_t)((0x100000000ull + w.band_count - 1) / w.band_count);
   k_xyz_tc<<<(unsigned)grid, kXyzThreads, smem, st>>>(spectral, n_pixels, w.band_count, nk, inv_bc, w.w32,
-                                                      1.0 / (double)spp, xyz, mode == 0 ? 3 : 1, status);
+                                                      1.0 / (double)spp, xyz, status);
 }
 
 }  // namespace srt
