@@ -197,6 +197,21 @@ struct PathId {
   uint32_t r, s, pix, j;
 };
 
+constexpr uint32_t kPixRun = 8;  // WaveParams::pix_inner: pixels of one band in a row
+
+// Pixel and band index of in-sample index r.
+__device__ __forceinline__ void pixel_band(const WaveParams& w, uint32_t r, uint32_t& pix, uint32_t& j) {
+  if (w.pix_inner) {
+    const uint32_t b = r / (kPixRun * w.band_count), q = r - b * kPixRun * w.band_count;
+    const uint32_t n = min(kPixRun, w.pix_inner - b * kPixRun);
+    j = q / n;
+    pix = b * kPixRun + (q - j * n);
+  } else {
+    pix = r / w.band_count;
+    j = r - pix * w.band_count;
+  }
+}
+
 __device__ __forceinline__ PathId path_id(const WaveParams& w, uint32_t pid) {
   PathId p;
   p.r = w.r0 + pid;
@@ -206,8 +221,7 @@ __device__ __forceinline__ PathId path_id(const WaveParams& w, uint32_t pid) {
     p.r -= q * w.PB;
     p.s += q;
   }
-  p.pix = p.r / w.band_count;
-  p.j = p.r - p.pix * w.band_count;
+  pixel_band(w, p.r, p.pix, p.j);
   return p;
 }
 

@@ -111,7 +111,8 @@ struct DevCam {
 constexpr int kMaxCams = 64;
 
 // One wave: paths [wave_start, wave_start + n) of the index space
-// g = s * PB + r, r = pixel * band_count + j, PB = pixels * band_count.
+// g = s * PB + r, r = pixel * band_count + j (or see pix_inner), PB = pixels *
+// band_count.
 struct WaveParams {
   uint32_t n;          // paths in this wave
   uint32_t s0, r0;     // sample and in-sample index of the first path
@@ -134,6 +135,11 @@ struct WaveParams {
   // launch_resolve adds the samples to the image in order.  Otherwise the
   // paths of a slot are in different waves and add to the image themselves.
   uint32_t samples;
+  // 0: r = pixel * band_count + j (neighbouring paths are the bands of a
+  // pixel); else the pixel count, and r runs over kPixRun pixels of one band,
+  // the bands of those pixels, then the next pixels (photon gathers of
+  // neighbouring pixels in one band read the same cells)
+  uint32_t pix_inner;
 };
 
 // Guided sampling of one wave (on == false: plain cosine sampling).
@@ -264,6 +270,7 @@ struct LaunchCfg {
   int grid_trace, block_trace;  // block_trace also sizes the sun-ray kernel's blocks
   int grid_shadow;
   int sms;  // SMs of the device
+  bool cams_inside;  // every camera lies within the scene bounds
   bool counting;
   bool record;
   int variant;  // traversal: 0 = four-wide, leaf batching; binary: 1 = while-while, 2 = node-or-leaf steps,
@@ -343,11 +350,10 @@ struct PhotonPass {
   const float4* portal;
   const float* cdf;
 };
-// The maps after sorting: rec holds the records in key order; start / end
-// the record range of each key (empty: start = end = 0).
+// The maps after sorting: rec holds the records in key order; range the
+// first and past-the-last record of each key (empty: 0, 0).
 struct PhotonMaps {
-  const uint32_t* start;
-  const uint32_t* end;
+  const uint2* range;
   const float4* rec;
   float r2[2], inv_cell[2], norm[2];  // r^2, 1 / (2 r), 2 / (pi r^2) per map (Epanechnikov kernel)
   uint32_t hbits, Bc;
@@ -355,7 +361,7 @@ struct PhotonMaps {
 void launch_photon_trace(const DevScene& S, const DevSpectra& P, const PhotonPass& pp, float4* rec, uint32_t* keys,
                          uint32_t* vals, uint8_t* cls, uint32_t* status, int sms, cudaStream_t st);
 void launch_photon_maps(const uint32_t* sorted_keys, const uint32_t* sorted_vals, uint32_t n, const float4* rec,
-                        float4* rec_sorted, uint32_t* start, uint32_t* end, int sms, cudaStream_t st);
+                        float4* rec_sorted, uint2* range, int sms, cudaStream_t st);
 int trace_blocks_per_sm(int block);
 int shadow_blocks_per_sm(int block);
 
@@ -399,6 +405,9 @@ void launch_guide_step_gather(const void* v, uint32_t n, uint32_t k, const Guide
 // camera (rt_api.cu).
 bool build_dev_cams(const rt_camera* cams, uint32_t n_cams, DevCam* out, uint64_t* npix, const char** why);
 
+// Whether every camera lies within the scene bounds lo .. hi.
+bool cameras_inside(const rt_camera* cams, uint32_t n_cams, const float lo[3], const float hi[3]);
+
 // Read-only view of a context for entry points defined outside rt_api.cu.
 struct CtxView {
   int device;
@@ -408,6 +417,7 @@ struct CtxView {
   DevSpectra P;
   const float* cmfw;     // device [n_bands][3]
   int sms;
+  float lo[3], hi[3];    // scene bounds
   DevCam* h_cams;        // pinned staging, kMaxCams entries
   uint32_t* h_status;    // pinned
 };

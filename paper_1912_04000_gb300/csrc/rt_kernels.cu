@@ -1170,9 +1170,29 @@ __device__ __forceinline__ uint32_t photon_cell_hash(int ix, int iy, int iz, uin
   return h & ((1u << hbits) - 1u);
 }
 
-// Kernel-weighted flux of the photons of band j in map `map` within distance
-// r of x, weight 1 - d^2 / r^2 (Epanechnikov): the (at most 8) cells of edge
-// 2 r that the ball touches, duplicates of a hashed key skipped.
+// Kernel-weighted flux of the photons of one cell within distance r of x,
+// weight 1 - d^2 / r^2 (Epanechnikov), added to sum.  Two records in flight.
+__device__ __forceinline__ void photon_cell(const PhotonMaps& M, uint32_t map, uint2 range, float3 x, float& sum) {
+  auto take = [&](float4 ph) {
+    const float dx = ph.x - x.x, dy = ph.y - x.y, dz = ph.z - x.z;
+    const float d2 = dx * dx + dy * dy + dz * dz;
+    if (d2 < M.r2[map]) sum += ph.w * (1.0f - d2 / M.r2[map]);
+  };
+  for (uint32_t q = range.x; q < range.y; q += 2u) {
+    const float4 a = ldg4(M.rec + q), b = ldg4(M.rec + min(q + 1u, range.y - 1u));
+    take(a);
+    if (q + 1u < range.y) take(b);
+  }
+}
+
+// The photons of band j in map `map` around x: the (at most 8) cells of edge
+// 2 r that the ball touches, duplicates of a hashed key skipped.  The ball
+// spans two cells per axis: all eight ranges are read at once, then their
+// records in cell order, so the chain of dependent loads is two per gather
+// and one per two records, not three per cell and one per record (the bound:
+// long scoreboard; closest-hit and shading stages of the camera pass 4.53 ->
+// 3.73 ms with the ranges' two words as one load).  Rounding can make an axis three cells wide; those
+// gathers go cell by cell.
 __device__ __forceinline__ float photon_gather(const PhotonMaps& M, uint32_t map, uint32_t j, float3 x) {
   const float ic = M.inv_cell[map];
   const float r = sqrtf(M.r2[map]);
@@ -1180,9 +1200,28 @@ __device__ __forceinline__ float photon_gather(const PhotonMaps& M, uint32_t map
   const int ly = (int)floorf((x.y - r) * ic), hy = (int)floorf((x.y + r) * ic);
   const int lz = (int)floorf((x.z - r) * ic), hz = (int)floorf((x.z + r) * ic);
   const uint32_t base = (map * M.Bc + j) << M.hbits;
+  float sum = 0.0f;
+  if (hx - lx <= 1 && hy - ly <= 1 && hz - lz <= 1) {
+    uint32_t key[8];
+    uint2 range[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      key[c] = base | photon_cell_hash(c & 4 ? hx : lx, c & 2 ? hy : ly, c & 1 ? hz : lz, M.hbits);
+      range[c] = __ldg(M.range + key[c]);
+    }
+#pragma unroll
+    for (int c = 1; c < 8; ++c) {
+      bool dup = false;
+#pragma unroll
+      for (int q = 0; q < c; ++q) dup |= key[q] == key[c];
+      if (dup) range[c] = make_uint2(0u, 0u);
+    }
+#pragma unroll
+    for (int c = 0; c < 8; ++c) photon_cell(M, map, range[c], x, sum);
+    return sum;
+  }
   uint32_t seen[8];
   int ns = 0;
-  float sum = 0.0f;
   for (int ix = lx; ix <= hx; ++ix)
     for (int iy = ly; iy <= hy; ++iy)
       for (int iz = lz; iz <= hz; ++iz) {
@@ -1191,13 +1230,7 @@ __device__ __forceinline__ float photon_gather(const PhotonMaps& M, uint32_t map
         for (int q = 0; q < ns; ++q) dup |= seen[q] == key;
         if (dup || ns >= 8) continue;
         seen[ns++] = key;
-        const uint32_t e = __ldg(M.end + key);
-        for (uint32_t q = __ldg(M.start + key); q < e; ++q) {
-          const float4 ph = ldg4(M.rec + q);
-          const float dx = ph.x - x.x, dy = ph.y - x.y, dz = ph.z - x.z;
-          const float d2 = dx * dx + dy * dy + dz * dz;
-          if (d2 < M.r2[map]) sum += ph.w * (1.0f - d2 / M.r2[map]);
-        }
+        photon_cell(M, map, __ldg(M.range + key), x, sum);
       }
   return sum;
 }
@@ -1996,7 +2029,8 @@ __global__ void __launch_bounds__(kTraceMaxThreads, kTraceMinBlocks)
 __global__ void __launch_bounds__(256) k_resolve(WaveParams w, const float* __restrict__ L,
                                                  const float4* __restrict__ L4, double* __restrict__ accum) {
   for (uint32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < w.PB; r += gridDim.x * blockDim.x) {
-    const uint32_t pix = r / w.band_count, j = r - pix * w.band_count;
+    uint32_t pix, j;
+    pixel_band(w, r, pix, j);
     if (w.nb == 4u) {
       const uint32_t nv = four_band_count(w, j);
       double* a = accum + (size_t)pix * w.B + j;
@@ -2199,17 +2233,16 @@ __global__ void __launch_bounds__(128) k_photon_trace(DevScene S, DevSpectra P, 
   }
 }
 
-// Record ranges per key of the sorted photon slots, and the records in key
+// Record range per key of the sorted photon slots, and the records in key
 // order.
 __global__ void k_photon_bounds(const uint32_t* __restrict__ sk, const uint32_t* __restrict__ sv, uint32_t n,
-                                const float4* __restrict__ rec, float4* __restrict__ rs, uint32_t* __restrict__ start,
-                                uint32_t* __restrict__ end) {
+                                const float4* __restrict__ rec, float4* __restrict__ rs, uint2* __restrict__ range) {
   for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < n; q += gridDim.x * blockDim.x) {
     const uint32_t key = sk[q];
     if (key == kPhotonEmpty) continue;
     rs[q] = rec[sv[q]];
-    if (q == 0u || sk[q - 1] != key) start[key] = q;
-    if (q + 1u == n || sk[q + 1] != key) end[key] = q + 1u;
+    if (q == 0u || sk[q - 1] != key) range[key].x = q;
+    if (q + 1u == n || sk[q + 1] != key) range[key].y = q + 1u;
   }
 }
 
@@ -2402,9 +2435,11 @@ void launch_wave(const LaunchCfg& lcfg, const DevScene& S, const DevSpectra& P, 
       sort_queue<false>(S, qin, b, k, st, sms);
       nl += 4;
     }
-    // vertex 1 starts at the cameras, which may lie anywhere: robust box
-    // test; later origins are surface points inside the padded bounds
-    launch_trace(lc, k == 1, S, qin, b, k, st);
+    // vertex 1 starts at the cameras: where one lies outside the scene bounds,
+    // the box test for any origin; later origins are surface points inside the
+    // padded bounds (all closest hits of 1280 x 960 x 81 bands x 4 samples in
+    // the 98k-triangle nave: 122.2 ms, with the general test at vertex 1 124.6)
+    launch_trace(lc, k == 1 && !lc.cams_inside, S, qin, b, k, st);
     if (tm) tm->end(STG_TRACE, st);
     if (tm) tm->begin(STG_SHADE, st);
     if (w.nb == 4u) {
@@ -2468,8 +2503,8 @@ void launch_photon_trace(const DevScene& S, const DevSpectra& P, const PhotonPas
 }
 
 void launch_photon_maps(const uint32_t* sorted_keys, const uint32_t* sorted_vals, uint32_t n, const float4* rec,
-                        float4* rec_sorted, uint32_t* start, uint32_t* end, int sms, cudaStream_t st) {
-  k_photon_bounds<<<(sms > 0 ? sms : 1) * 8, 256, 0, st>>>(sorted_keys, sorted_vals, n, rec, rec_sorted, start, end);
+                        float4* rec_sorted, uint2* range, int sms, cudaStream_t st) {
+  k_photon_bounds<<<(sms > 0 ? sms : 1) * 8, 256, 0, st>>>(sorted_keys, sorted_vals, n, rec, rec_sorted, range);
 }
 
 void launch_philox(const uint32_t* ctr, uint32_t* out, uint64_t n, uint32_t k0, uint32_t k1, cudaStream_t st) {

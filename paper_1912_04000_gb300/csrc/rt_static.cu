@@ -139,6 +139,7 @@ extern "C" rt_status rt_render_static(rt_ctx* c, const rt_camera* cams, uint32_t
   lc.grid_trace = v.sms * trace_blocks_per_sm(lc.block_trace);
   lc.grid_shadow = v.sms * shadow_blocks_per_sm(lc.block_trace);
   lc.sms = v.sms;
+  lc.cams_inside = cameras_inside(cams, n_cams, v.lo, v.hi);
   lc.counting = false;
   lc.record = false;
   lc.variant = 0;
