@@ -77,7 +77,7 @@ struct rt_ctx {
   size_t accum_cap = 0;
   float* d_xyz = nullptr;
   size_t xyz_cap = 0;
-  uint32_t* h_status = nullptr;  // pinned
+  uint32_t* h_status = nullptr;  // pinned: status word, a batch's loss
   Totals* h_tot = nullptr;       // pinned
   uint32_t* d_status_aux = nullptr;
   cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
@@ -319,7 +319,7 @@ rt_status rt_create(int device, void* cuda_stream, rt_ctx** out) {
       cudaMalloc(&c->wb.status, sizeof(uint32_t)) != cudaSuccess ||
       cudaMalloc(&c->d_cams, sizeof(DevCam) * kMaxCams) != cudaSuccess ||
       cudaMallocHost(&c->h_cams, sizeof(DevCam) * kMaxCams) != cudaSuccess ||
-      cudaMallocHost(&c->h_status, sizeof(uint32_t)) != cudaSuccess ||
+      cudaMallocHost(&c->h_status, 2 * sizeof(uint32_t)) != cudaSuccess ||
       cudaMallocHost(&c->h_tot, sizeof(Totals)) != cudaSuccess) {
     rt_destroy(c);
     return RT_ERR_OOM;
@@ -1404,7 +1404,7 @@ rt_status rt_guide_init(rt_ctx* c, const rt_guide_config* cfg_in, uint64_t seed)
     CUDA_TRY(c, cudaMalloc(&G.vW, guide_wcount() * 4));
     CUDA_TRY(c, cudaMalloc(&G.dW, guide_wcount() * 4));
     CUDA_TRY(c, cudaMalloc(&G.dWpart, (size_t)c->sms * guide_wcount() * 4));
-    CUDA_TRY(c, cudaMalloc(&G.scratch, 64));
+    CUDA_TRY(c, cudaMalloc(&G.scratch, (16 + 2 * kGuideChunks) * 4));  // sums, then per-chunk words
     CUDA_TRY(c, cudaMalloc(&G.pack, guide_wpack_bytes()));
   }
   G.cfg = cfg;
@@ -1480,14 +1480,13 @@ rt_status rt_guide_eval(rt_ctx* c, const float* rec_dev, uint64_t n, float* Y_de
   return status_to_rt(c, *c->h_status);
 }
 
-// Gradient of one batch into G.dgrid / G.dW (enqueued, no synchronisation).
-static void guide_grad_enqueue(rt_ctx* c, const float* rec_dev, uint64_t n) {
+// Gradient of one batch into dgrid (16-byte aligned) and dW (enqueued, no
+// synchronisation).
+static void guide_grad_enqueue(rt_ctx* c, const float* rec_dev, uint64_t n, float* dgrid, float* dW) {
   auto& G = c->guide;
-  cudaMemsetAsync(G.dgrid, 0, G.n_grid * 4, c->stream);
-  cudaMemsetAsync(G.dW, 0, guide_wcount() * 4, c->stream);
-  cudaMemsetAsync(G.scratch, 0, 64, c->stream);
-  launch_guide_train(G.dev, G.pack, rec_dev, n, G.scratch, G.dW, G.dWpart, G.dgrid, G.scratch + 1, c->wb.status, c->sms,
-                     c->stream);
+  cudaMemsetAsync(dgrid, 0, G.n_grid * 4, c->stream);
+  launch_guide_train(G.dev, G.pack, rec_dev, n, G.scratch + 16, dW, G.dWpart, dgrid, G.scratch + 1, c->wb.status,
+                     c->sms, c->stream);
 }
 
 // Adam step on the gradient in G.dgrid / G.dW, then repack the BF16 weights.
@@ -1504,18 +1503,20 @@ static void guide_update_enqueue(rt_ctx* c) {
 }
 
 static void guide_train_enqueue(rt_ctx* c, const float* rec, uint64_t n) {
-  guide_grad_enqueue(c, rec, n);
+  guide_grad_enqueue(c, rec, n, c->guide.dgrid, c->guide.dW);
   guide_update_enqueue(c);
 }
 
-static rt_status guide_grad_impl(rt_ctx* c, const float* rec_dev, uint64_t n, float* loss_host) {
+static rt_status guide_grad_impl(rt_ctx* c, const float* rec_dev, uint64_t n, float* loss_host, float* dgrid,
+                                 float* dW) {
   auto& G = c->guide;
   CUDA_TRY(c, cudaMemsetAsync(c->wb.status, 0, 4, c->stream));
-  guide_grad_enqueue(c, rec_dev, n);
+  guide_grad_enqueue(c, rec_dev, n, dgrid, dW);
   CUDA_TRY(c, cudaGetLastError());
-  if (loss_host) CUDA_TRY(c, cudaMemcpyAsync(loss_host, G.scratch + 1, 4, cudaMemcpyDeviceToHost, c->stream));
+  if (loss_host) CUDA_TRY(c, cudaMemcpyAsync(c->h_status + 1, G.scratch + 1, 4, cudaMemcpyDeviceToHost, c->stream));
   CUDA_TRY(c, cudaMemcpyAsync(c->h_status, c->wb.status, 4, cudaMemcpyDeviceToHost, c->stream));
   CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+  if (loss_host) std::memcpy(loss_host, c->h_status + 1, 4);
   return status_to_rt(c, *c->h_status);
 }
 
@@ -1524,11 +1525,16 @@ rt_status rt_guide_grad(rt_ctx* c, const float* rec_dev, uint64_t n, float* loss
   if (!rec_dev || n == 0) return fail(c, RT_ERR_ARG, "rt_guide_grad: no records");
   if (((uintptr_t)rec_dev & 15u) != 0) return fail(c, RT_ERR_ARG, "rt_guide_grad: records must be 16-byte aligned");
   cudaSetDevice(c->device);
-  if (rt_status e = guide_grad_impl(c, rec_dev, n, loss)) return e;
   auto& G = c->guide;
-  if (dgrid_dev) CUDA_TRY(c, cudaMemcpyAsync(dgrid_dev, G.dgrid, G.n_grid * 4, cudaMemcpyDeviceToDevice, c->stream));
-  if (dW_dev) CUDA_TRY(c, cudaMemcpyAsync(dW_dev, G.dW, guide_wcount() * 4, cudaMemcpyDeviceToDevice, c->stream));
-  CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+  // the kernels add to the caller's grid gradient where their 16-byte adds
+  // can (a copy of 2^22 entries takes 20 us, a tenth of a batch of 524,288
+  // records), else to the guide's own and copy
+  const bool direct = dgrid_dev && ((uintptr_t)dgrid_dev & 15u) == 0;
+  if (rt_status e = guide_grad_impl(c, rec_dev, n, loss, direct ? dgrid_dev : G.dgrid, dW_dev ? dW_dev : G.dW)) return e;
+  if (dgrid_dev && !direct) {
+    CUDA_TRY(c, cudaMemcpyAsync(dgrid_dev, G.dgrid, G.n_grid * 4, cudaMemcpyDeviceToDevice, c->stream));
+    CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+  }
   return RT_OK;
 }
 
@@ -1538,7 +1544,7 @@ rt_status rt_guide_train_step(rt_ctx* c, const float* rec_dev, uint64_t n, float
   if (((uintptr_t)rec_dev & 15u) != 0)
     return fail(c, RT_ERR_ARG, "rt_guide_train_step: records must be 16-byte aligned");
   cudaSetDevice(c->device);
-  if (rt_status e = guide_grad_impl(c, rec_dev, n, loss)) return e;
+  if (rt_status e = guide_grad_impl(c, rec_dev, n, loss, c->guide.dgrid, c->guide.dW)) return e;
   guide_update_enqueue(c);
   CUDA_TRY(c, cudaGetLastError());
   CUDA_TRY(c, cudaStreamSynchronize(c->stream));

@@ -371,13 +371,14 @@ __device__ __forceinline__ void corner_weights(const float fr[3], float w[8]) {
   for (int k = 0; k < 8; ++k) w[k] = wxy[k & 3] * wz[k >> 2];
 }
 
-// Hash-grid features of levels l0 .. l0 + 3, 16 values (the arithmetic of
+// Hash-grid features of levels l0 .. l0 + N - 1, 4 N values (the arithmetic of
 // encode()); res: the per-level resolutions, staged in shared memory.
-__device__ __forceinline__ void encode_levels4(const GuideDev& g, const uint32_t* res, const float u[3], int l0,
-                                               float* f) {
+template <int N>
+__device__ __forceinline__ void encode_levels(const GuideDev& g, const uint32_t* res, const float u[3], int l0,
+                                              float* f) {
   const uint32_t T = 1u << g.log2T;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < N; ++i) {
     const int l = l0 + i;
     const float rl = (float)res[l];
     uint32_t c[3];
@@ -413,18 +414,23 @@ __device__ __forceinline__ void encode_levels4(const GuideDev& g, const uint32_t
 // ---------------------------------------------------------------------------
 // training: forward, loss gradient, backward, gradient accumulation
 // ---------------------------------------------------------------------------
-// A CTA of 256 threads serves 128 records per tile, two threads per record
-// (half h = t / 128; threads t and t + 128 share a TMEM lane).  Records of
-// zero weight add nothing to the loss or its gradient and are skipped: each
-// CTA walks a contiguous chunk of the batch, four records per thread and
-// round, and compacts the indices of the weighted records into full tiles.
+// A CTA of 512 threads serves 128 records per tile, four threads per record
+// (part h = t / 128; threads t, t + 128, .. share a TMEM lane).  Records of
+// zero weight add nothing to the loss or its gradient and are skipped:
+// k_guide_count counts the weighted records of each chunk of the batch, a CTA
+// takes its even share of them, in batch order, and compacts their indices
+// into full tiles.
+// Bound by the requests to L2: 64 gathers and 64 adds of 16 bytes per record,
+// 6.4 million for 52,400 weighted records of 524,288, in two bursts per tile;
+// 105 us (126 with two threads per record and equal parts of the batch, whose
+// fullest parts took a fourth tile).
 // Weight gradients dW_l = H_{l-1}^T dZ_l use A' = [H_{l-1}^T; 0] (M = 128)
 // and B' = dZ_l^T, both made from the K-major activation tiles by 8 x 8
 // transposes (ldmatrix / stmatrix.trans), and accumulate in TMEM over all
 // tiles of the CTA; each CTA then stores its sums as one partial (layer l's
 // block column-major: element (in, o) at w_off(l) + 64 o + in) and
 // k_dw_reduce adds the partials in a fixed order.
-constexpr int kTrainThreads = 2 * kRows;
+constexpr int kTrainThreads = 4 * kRows;
 constexpr uint32_t kTrX = kWPack;
 constexpr uint32_t kTrH1 = kTrX + kATileB;
 constexpr uint32_t kTrH2 = kTrH1 + kATileB;
@@ -432,11 +438,16 @@ constexpr uint32_t kTrH3 = kTrH2 + kATileB;
 constexpr uint32_t kTrDZ = kTrH3 + kATileB;
 constexpr uint32_t kTrAp = kTrDZ + kATileB;           // [128 x 128] = 32 KB
 constexpr uint32_t kTrBp = kTrAp + 8 * kSliceA;       // <= [64 x 128] = 16 KB
-constexpr uint32_t kTrScan = 4;                       // records per thread and scan round
-constexpr uint32_t kTrListN = kRows + kTrScan * kTrainThreads;  // a short tile + one round
-constexpr uint32_t kTrList = kTrBp + 8 * 64 * 32;     // record indices
-constexpr uint32_t kTrMisc = kTrList + kTrListN * 4;
-constexpr uint32_t kTrainSmem = kTrMisc + 128;
+constexpr uint32_t kTrScan = 2;                       // records per thread and scan round
+constexpr uint32_t kTrRound = kTrScan * kTrainThreads;
+constexpr uint32_t kTrListN = kRows + kTrRound;       // a short tile + one round
+constexpr uint32_t kTrList = kTrBp + 8 * 64 * 32;     // record indices (64-bit)
+constexpr uint32_t kTrMaxChunks = kGuideChunks;       // chunks of the batch
+static_assert(kTrMaxChunks == 2 * kTrainThreads, "two chunk counts per thread");
+constexpr uint32_t kTrPre = kTrList + kTrListN * 8;   // weighted records before each chunk (64-bit)
+constexpr uint32_t kTrXch = kTrPre + kTrMaxChunks * 8;  // head exchange, 12 floats per record
+constexpr uint32_t kTrMisc = kTrXch + kRows * 12 * 4;
+constexpr uint32_t kTrainSmem = kTrMisc + 512;
 static_assert(kTrainSmem <= 227 * 1024, "training kernel shared memory");
 
 __device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t& a, uint32_t& b, uint32_t& c, uint32_t& d) {
@@ -476,21 +487,68 @@ __device__ __forceinline__ void transpose_tile(const unsigned char* src, unsigne
   }
 }
 
+// Weighted records and weight sum of each chunk of the batch (chunk records,
+// a multiple of kTrRound; one block per chunk).  The strided reads fetch a
+// 32-byte sector per 48-byte record: 16.8 MB for 524,288 records, 6.7 us (12.0
+// by warps that added to one word).  Also clears the loss.
+__global__ void __launch_bounds__(256) k_guide_count(const float4* __restrict__ rec, uint64_t n, uint64_t chunk,
+                                                     uint32_t* __restrict__ cnt, float* __restrict__ wsum,
+                                                     float* __restrict__ loss) {
+  __shared__ float ss[8];
+  __shared__ uint32_t sc[8];
+  const uint64_t c0 = blockIdx.x * chunk, c1 = min(c0 + chunk, n);
+  float s = 0.0f;
+  uint32_t c = 0;
+  for (uint64_t i = c0 + threadIdx.x; i < c1; i += 4u * 256u) {
+    float w[4];
+#pragma unroll
+    for (uint32_t q = 0; q < 4u; ++q) w[q] = i + 256u * q < c1 ? __ldg((const float*)(rec + 3 * (i + 256u * q)) + 3) : 0.0f;
+#pragma unroll
+    for (uint32_t q = 0; q < 4u; ++q) {
+      s += w[q];
+      c += w[q] > 0.0f ? 1u : 0u;
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    s += __shfl_xor_sync(0xffffffffu, s, o);
+    c += __shfl_xor_sync(0xffffffffu, c, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    ss[threadIdx.x >> 5] = s;
+    sc[threadIdx.x >> 5] = c;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) {
+      s += ss[w];
+      c += sc[w];
+    }
+    cnt[blockIdx.x] = c;
+    wsum[blockIdx.x] = s;
+    if (blockIdx.x == 0) *loss = 0.0f;
+  }
+}
+
 __global__ void __launch_bounds__(kTrainThreads, 1)
     k_guide_train(GuideDev g, const uint4* __restrict__ wpack, const float4* __restrict__ rec, uint64_t n,
-                  const float* __restrict__ wsum, float* __restrict__ dWpart, float* __restrict__ dgrid,
-                  float* __restrict__ loss, uint32_t* status) {
+                  uint64_t chunk, uint32_t nchunks, const uint32_t* __restrict__ ccnt, const float* __restrict__ cwsum,
+                  float* __restrict__ dWpart, float* __restrict__ dgrid, float* __restrict__ loss, uint32_t* status) {
   extern __shared__ __align__(1024) unsigned char smem[];
   unsigned char* AX = smem + kTrX;
   unsigned char* ADZ = smem + kTrDZ;
   unsigned char* Ap = smem + kTrAp;
   unsigned char* Bp = smem + kTrBp;
-  uint32_t* list = (uint32_t*)(smem + kTrList);
+  uint64_t* list = (uint64_t*)(smem + kTrList);
+  uint64_t* pre = (uint64_t*)(smem + kTrPre);
+  float* xch = (float*)(smem + kTrXch);
   uint64_t* mbar = (uint64_t*)(smem + kTrMisc);
-  uint32_t* tslot = (uint32_t*)(mbar + 1);
+  constexpr uint32_t kWarps = kTrainThreads / 32;
+  uint64_t* wtot = mbar + 1;                     // [kWarps] per-warp chunk counts
+  uint32_t* tslot = (uint32_t*)(wtot + kWarps);
   float* lsum = (float*)(tslot + 1);
-  uint32_t* wcnt = (uint32_t*)(lsum + 1);  // [8] per-warp counts, [8] list length
-  uint32_t* sres = wcnt + 9;               // [kLevels] grid resolutions
+  float* wwgt = lsum + 1;                        // [kWarps] per-warp weight sums
+  uint32_t* wcnt = (uint32_t*)(wwgt + kWarps);   // [kWarps] per-warp counts
+  uint32_t* sres = wcnt + kWarps;                // [kLevels] grid resolutions
   const uint32_t tid = threadIdx.x, warp = tid >> 5, lane = tid & 31u;
   const uint32_t r = tid & (kRows - 1), h = tid >> 7;
   load_weights(smem, wpack);
@@ -503,9 +561,23 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
     tc_mbar_init(mbar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     *lsum = 0.0f;
-    wcnt[8] = 0u;
   }
   if (warp == 0) tc_tmem_alloc(tslot, 512);
+  // prefix of the chunks' counts, the total weight (the same order in every CTA)
+  const uint32_t k0 = 2u * tid;
+  const uint32_t n0 = k0 < nchunks ? __ldg(ccnt + k0) : 0u, n1 = k0 + 1u < nchunks ? __ldg(ccnt + k0 + 1u) : 0u;
+  float ws = (k0 < nchunks ? __ldg(cwsum + k0) : 0.0f) + (k0 + 1u < nchunks ? __ldg(cwsum + k0 + 1u) : 0.0f);
+  uint64_t incl0 = (uint64_t)n0 + n1;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint64_t v = __shfl_up_sync(0xffffffffu, incl0, o);
+    if (lane >= (uint32_t)o) incl0 += v;
+    ws += __shfl_xor_sync(0xffffffffu, ws, o);
+  }
+  if (lane == 31) {
+    wtot[warp] = incl0;
+    wwgt[warp] = ws;
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -513,23 +585,39 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
   const uint32_t trow = tmem + (((warp & 3u) * 32u) << 16);
   Sync sy{mbar, 0u, true};
   const uint32_t id64 = tc_idesc_bf16(kRows, 64), id48 = tc_idesc_bf16(kRows, kOut);
-  const float total = *wsum;
-  const uint64_t per = (n + gridDim.x - 1) / gridDim.x;
-  const uint64_t c0 = min((uint64_t)blockIdx.x * per, n), c1 = min(c0 + per, n);
-  uint64_t cur = c0;
+  float total = 0.0f;
+  uint64_t weighted = 0, before = incl0 - n0 - n1;
+  for (uint32_t w2 = 0; w2 < kWarps; ++w2) {
+    if (w2 < warp) before += wtot[w2];
+    weighted += wtot[w2];
+    total += wwgt[w2];
+  }
+  pre[k0] = before;
+  pre[k0 + 1u] = before + n0;
+  __syncthreads();
+  // this CTA's share of the weighted records: numbers lo .. lo + left - 1
+  // (an even share: 345 of 52,400 in three tiles each; equal parts of the
+  // batch gave two CTAs a fourth tile, a quarter of the kernel's time)
+  const uint64_t lo = weighted / gridDim.x * blockIdx.x + min((uint64_t)blockIdx.x, weighted % gridDim.x);
+  uint64_t left = weighted / gridDim.x + (blockIdx.x < weighted % gridDim.x ? 1u : 0u);
+  uint32_t ch = 0;  // last chunk that starts at or before lo
+  for (uint32_t step = kTrMaxChunks / 2u; step > 0u; step >>= 1)
+    if (ch + step < nchunks && pre[ch + step] <= lo) ch += step;
+  uint64_t cur = ch * chunk, skip = lo - pre[ch];
+  uint32_t nlist = 0;
   bool first = true;
   float my_loss = 0.0f;
   while (sy.ok) {
     // compact the indices of weighted records until a tile is full
-    uint32_t nl = wcnt[8];
-    while (nl < (uint32_t)kRows && cur < c1) {
-      // records cur + tid + 256 q, q < 4: independent loads, one scan
+    uint32_t nl = nlist;
+    while (nl < (uint32_t)kRows && left > 0 && cur < n) {
+      // records cur + tid + 512 q, q < 2: independent loads, one scan
       bool take[kTrScan];
       uint32_t cnt_t = 0;
 #pragma unroll
       for (uint32_t q = 0; q < kTrScan; ++q) {
         const uint64_t i = cur + tid + (uint64_t)q * kTrainThreads;
-        take[q] = i < c1 && __ldg((const float*)(rec + 3 * i) + 3) > 0.0f;
+        take[q] = i < n && __ldg((const float*)(rec + 3 * i) + 3) > 0.0f;
         cnt_t += take[q] ? 1u : 0u;
       }
       uint32_t incl = cnt_t;
@@ -540,26 +628,33 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
       }
       if (lane == 31) wcnt[warp] = incl;
       __syncthreads();
-      uint32_t off = nl + incl - cnt_t;
-      for (uint32_t w2 = 0; w2 < warp; ++w2) off += wcnt[w2];
+      uint32_t at = incl - cnt_t, tot = 0;
+#pragma unroll
+      for (uint32_t w2 = 0; w2 < kWarps; ++w2) {
+        if (w2 < warp) at += wcnt[w2];
+        tot += wcnt[w2];
+      }
+      // drop the records of the CTAs before this one and after it
+      const uint32_t drop = (uint32_t)min((uint64_t)tot, skip), use = (uint32_t)min((uint64_t)(tot - drop), left);
 #pragma unroll
       for (uint32_t q = 0; q < kTrScan; ++q)
-        if (take[q]) list[off++] = (uint32_t)(cur + tid + (uint64_t)q * kTrainThreads - c0);
-      uint32_t tot = 0;
-      for (uint32_t w2 = 0; w2 < (blockDim.x >> 5); ++w2) tot += wcnt[w2];
+        if (take[q]) {
+          if (at >= drop && at - drop < use) list[nl + at - drop] = cur + tid + (uint64_t)q * kTrainThreads;
+          ++at;
+        }
       __syncthreads();
-      nl += tot;
-      cur += (uint64_t)kTrScan * kTrainThreads;
+      nl += use;
+      left -= use;
+      skip -= drop;
+      cur += kTrRound;
     }
     if (nl == 0) break;
     const uint32_t nt = min(nl, (uint32_t)kRows);
     const bool valid = r < nt;
-    const uint64_t ri = valid ? c0 + list[r] : 0;
     Rec rc{};
-    if (valid) rc = load_rec(rec, ri);
+    if (valid) rc = load_rec(rec, list[r]);
     // carry the surplus indices over to the next tile
-    __syncthreads();
-    uint32_t carry[kTrScan];
+    uint64_t carry[kTrScan];
 #pragma unroll
     for (uint32_t q = 0; q < kTrScan; ++q) {
       const uint32_t t = tid + q * kTrainThreads;
@@ -571,85 +666,105 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
       const uint32_t t = tid + q * kTrainThreads;
       if (t < nl - nt) list[t] = carry[q];
     }
-    if (tid == 0) wcnt[8] = nl - nt;
-    // encoding: half 0 grid levels 0-3 and SH, half 1 levels 4-7 and group
+    nlist = nl - nt;
+    // encoding: part h grid levels 2h, 2h + 1 and eight columns of the SH
+    // (h < 2) or the group
     {
-      float u[3], f[16];
+      float u[3], f[8];
       unit_pos(g, rc.p, u);
       if (valid) {
-        encode_levels4(g, sres, u, 4 * (int)h, f);
+        encode_levels<2>(g, sres, u, 2 * (int)h, f);
       } else {
 #pragma unroll
-        for (int c = 0; c < 16; ++c) f[c] = 0.0f;
+        for (int c = 0; c < 8; ++c) f[c] = 0.0f;
       }
-      put8(AX, r, 16 * (int)h, f);
-      put8(AX, r, 16 * (int)h + 8, f + 8);
-      if (h == 0) {
-        if (valid) sh16(rc.n.x, rc.n.y, rc.n.z, f);
-        put8(AX, r, 32, f);
-        put8(AX, r, 40, f + 8);
+      put8(AX, r, 8 * (int)h, f);
+      if (h < 2u) {
+        float sh[16];
+        sh16(rc.n.x, rc.n.y, rc.n.z, sh);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) f[c] = valid ? (h ? sh[8 + c] : sh[c]) : 0.0f;
       } else {
 #pragma unroll
-        for (int c = 0; c < 16; ++c) f[c] = (valid && (uint32_t)c == rc.group) ? 1.0f : 0.0f;
-        put8(AX, r, 48, f);
-        put8(AX, r, 56, f + 8);
+        for (int c = 0; c < 8; ++c) f[c] = (valid && (uint32_t)c + 8u * (h - 2u) == rc.group) ? 1.0f : 0.0f;
       }
+      put8(AX, r, 32 + 8 * (int)h, f);
     }
     // forward
     for (int l = 0; l < 3; ++l) {
       publish();
       if (tid == 0) gemm(tmem, smem + kTrX + kATileB * (uint32_t)l, kSliceA, smem + wf_off(l), 2048, 4, id64, false);
       mma_wait(sy, status);
-      float v[32];
-      tc_tmem_ld16x2(trow + 32u * h, v);
+      float v[16];
+      tc_tmem_ld16(trow + 16u * h, v);
       unsigned char* Hl = smem + kTrH1 + kATileB * (uint32_t)l;
 #pragma unroll
-      for (int c = 0; c < 32; c += 8) {
-        float t[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) t[e] = fmaxf(v[c + e], 0.0f);
-        put8(Hl, r, 32 * (int)h + c, t);
-      }
+      for (int c = 0; c < 16; ++c) v[c] = fmaxf(v[c], 0.0f);
+      put8(Hl, r, 16 * (int)h, v);
+      put8(Hl, r, 16 * (int)h + 8, v + 8);
     }
     publish();
     if (tid == 0) gemm(tmem, smem + kTrH3, kSliceA, smem + wf_off(3), kOut * 32, 4, id48, false);
     mma_wait(sy, status);
-    // head (half 0): loss and dL/dY, written as dZ_3 into ADZ
-    if (h == 0) {
-      float y[48];
-      tc_tmem_ld16x2(trow, y);
-      tc_tmem_ld16(trow + 32u, y + 32);
+    // head: loss and dL/dY, written as dZ_3 into ADZ.  Part h owns lobes
+    // 2h, 2h + 1 (Y[10h .. 10h + 9]); the softmax maximum and sum and the
+    // density are exchanged through shared memory.
+    {
+      float yv[32], y[10];
+      tc_tmem_ld16x2(trow + 16u * (h >> 1), yv);
+#pragma unroll
+      for (int c = 0; c < 10; ++c) y[c] = h == 0u ? yv[c] : h == 1u ? yv[c + 10] : h == 2u ? yv[c + 4] : yv[c + 14];
+      float* X = xch + r * 12u;
+      X[h] = fmaxf(y[0], y[5]);
+      __syncthreads();
+      const float mx = fmaxf(fmaxf(X[0], X[1]), fmaxf(X[2], X[3]));
+      float pi[2] = {expf(y[0] - mx), expf(y[5] - mx)};
+      X[4 + h] = pi[0] + pi[1];
+      __syncthreads();
+      const float is = 1.0f / ((X[4] + X[5]) + (X[6] + X[7]));
+      float mu[2][3], nrm[2], kap[2], pj[2], q = 0.0f;
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        pi[j] *= is;
+        const float m0 = y[5 * j + 1], m1 = y[5 * j + 2], m2 = y[5 * j + 3];
+        nrm[j] = fmaxf(sqrtf(m0 * m0 + m1 * m1 + m2 * m2), 1e-6f);
+        mu[j][0] = m0 / nrm[j];
+        mu[j][1] = m1 / nrm[j];
+        mu[j][2] = m2 / nrm[j];
+        kap[j] = 0.5f + softplusf(y[5 * j + 4]);
+        pj[j] = vmf_pdf(kap[j], mu[j], rc.w);
+        q += pi[j] * pj[j];
+      }
+      X[8 + h] = q;
+      __syncthreads();
+      q = (X[8] + X[9]) + (X[10] + X[11]);
       const float a = (valid && total > 0.0f) ? rc.weight / total : 0.0f;
-      float dY[kOut];
+      float dY[10];
 #pragma unroll
-      for (int c = 0; c < kOut; ++c) dY[c] = 0.0f;
+      for (int c = 0; c < 10; ++c) dY[c] = 0.0f;
       if (a > 0.0f) {
-        Mix mx;
-        mixture(y, mx);
-        float pj[kLobes], q = 0.0f;
-#pragma unroll
-        for (int j = 0; j < kLobes; ++j) {
-          pj[j] = vmf_pdf(mx.kappa[j], mx.mu[j], rc.w);
-          q += mx.pi[j] * pj[j];
-        }
-        my_loss -= a * logf(q);
+        if (h == 0u) my_loss -= a * logf(q);
         const float3 w = rc.w;
 #pragma unroll
-        for (int j = 0; j < kLobes; ++j) {
-          const float rj = mx.pi[j] * pj[j] / q;
-          const float c = mx.mu[j][0] * w.x + mx.mu[j][1] * w.y + mx.mu[j][2] * w.z;
-          dY[5 * j] = -a * (rj - mx.pi[j]);
-          const float fj = -a * rj * mx.kappa[j] / mx.mnorm[j];
-          dY[5 * j + 1] = fj * (w.x - c * mx.mu[j][0]);
-          dY[5 * j + 2] = fj * (w.y - c * mx.mu[j][1]);
-          dY[5 * j + 3] = fj * (w.z - c * mx.mu[j][2]);
-          const float k = mx.kappa[j];
+        for (int j = 0; j < 2; ++j) {
+          const float rj = pi[j] * pj[j] / q;
+          const float c = mu[j][0] * w.x + mu[j][1] * w.y + mu[j][2] * w.z;
+          dY[5 * j] = -a * (rj - pi[j]);
+          const float fj = -a * rj * kap[j] / nrm[j];
+          dY[5 * j + 1] = fj * (w.x - c * mu[j][0]);
+          dY[5 * j + 2] = fj * (w.y - c * mu[j][1]);
+          dY[5 * j + 3] = fj * (w.z - c * mu[j][2]);
+          const float k = kap[j];
           const float dlogp = 1.0f / k - 2.0f / expm1f(2.0f * k) + (c - 1.0f);
           dY[5 * j + 4] = -a * rj * dlogp / (1.0f + expf(-y[5 * j + 4]));
         }
       }
 #pragma unroll
-      for (int c = 0; c < kOut; c += 8) put8(ADZ, r, c, dY + c);
+      for (int c = 0; c < 10; c += 2) {
+        const uint32_t col = 10u * h + (uint32_t)c;
+        *(uint32_t*)(ADZ + (col >> 4) * kSliceA + tc_kmajor_off(r, col & 15u)) = tc_bf16x2_bits(dY[c], dY[c + 1]);
+      }
+      if (h == 3u) *(uint4*)(ADZ + 2u * kSliceA + tc_kmajor_off(r, 8u)) = make_uint4(0u, 0u, 0u, 0u);
     }
     // backward: layer l = 3 (W4, out 48) down to 0 (W1)
     for (int l = 3; l >= 0; --l) {
@@ -670,12 +785,12 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
       mma_wait(sy, status);
       if (l > 0) {
         // dZ_{l-1} = dH_{l-1} where the forward activation was positive
-        float v[32];
-        tc_tmem_ld16x2(trow + 32u * h, v);
+        float v[16];
+        tc_tmem_ld16(trow + 16u * h, v);
         const unsigned char* Hm = smem + kTrX + kATileB * (uint32_t)l;
 #pragma unroll
-        for (int c = 0; c < 32; c += 8) {
-          const int col = 32 * (int)h + c;
+        for (int c = 0; c < 16; c += 8) {
+          const int col = 16 * (int)h + c;
           const uint4 hb = *(const uint4*)(Hm + (col >> 4) * kSliceA + tc_kmajor_off(r, (uint32_t)(col & 15)));
           const uint32_t hw[4] = {hb.x, hb.y, hb.z, hb.w};
           float t[8];
@@ -687,16 +802,18 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
           put8(ADZ, r, col, t);
         }
       } else {
-        // dX of grid levels 4h .. 4h + 3 -> grid gradient
-        float dx[16];
-        tc_tmem_ld16(trow + 16u * h, dx);
+        // dX of grid levels 2h, 2h + 1 -> grid gradient
+        float dv[16], dx[8];
+        tc_tmem_ld16(trow + 16u * (h >> 1), dv);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) dx[c] = h & 1u ? dv[c + 8] : dv[c];
         if (valid && rc.weight > 0.0f && total > 0.0f) {
           float u[3];
           unit_pos(g, rc.p, u);
           const uint32_t T = 1u << g.log2T;
-#pragma unroll 1
-          for (int i = 0; i < 4; ++i) {
-            const int l2 = 4 * (int)h + i;
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            const int l2 = 2 * (int)h + i;
             const float d0 = dx[4 * i], d1 = dx[4 * i + 1], d2 = dx[4 * i + 2], d3 = dx[4 * i + 3];
             if (d0 == 0.0f && d1 == 0.0f && d2 == 0.0f && d3 == 0.0f) continue;
             const float rl = (float)sres[l2];
@@ -722,25 +839,21 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
     }
     first = false;
   }
-  // accumulated weight gradients: TMEM lanes 0..63 (warps 0, 1, 4, 5) =
+  // accumulated weight gradients: TMEM lanes 0..63 (warps w, w % 4 < 2) =
   // input rows; this CTA's partial, element (in, o) of layer l at
-  // w_off(l) + 64 o + in (a warp stores 32 consecutive floats per column)
+  // w_off(l) + 64 o + in (a warp stores 32 consecutive floats per column);
+  // part h columns 16h .. 16h + 15
   float* part = dWpart + (size_t)blockIdx.x * kWSize;
   if (!first && sy.ok) {
     if ((warp & 3u) < 2u) {
       const uint32_t in = (warp & 1u) * 32u + lane;
       for (int l = 0; l < 4; ++l) {
-        const int out = layer_out(l);
-        float row[32];
-        // half 0 columns 0..31, half 1 columns 32..out-1
-        const int o0 = 32 * (int)h, nc = min(32, out - o0);
-        const uint32_t col0 = 64u * (uint32_t)(l + 1) + (uint32_t)o0;
-        if (nc == 32) {
-          tc_tmem_ld16x2(trow + col0, row);
-        } else {
-          tc_tmem_ld16(trow + col0, row);
-        }
-        for (int o = 0; o < nc; ++o) part[w_off(l) + 64 * (o0 + o) + in] = row[o];
+        const int o0 = 16 * (int)h;
+        if (o0 >= layer_out(l)) continue;
+        float row[16];
+        tc_tmem_ld16(trow + 64u * (uint32_t)(l + 1) + (uint32_t)o0, row);
+#pragma unroll
+        for (int o = 0; o < 16; ++o) part[w_off(l) + 64 * (o0 + o) + in] = row[o];
       }
     }
   } else {
@@ -755,16 +868,8 @@ __global__ void __launch_bounds__(kTrainThreads, 1)
 }
 
 // ---------------------------------------------------------------------------
-// small kernels: weight sum, Adam, BF16 packing, initialisation
+// small kernels: Adam, BF16 packing, initialisation
 // ---------------------------------------------------------------------------
-__global__ void k_weight_sum(const float4* __restrict__ rec, uint64_t n, float* out) {
-  float s = 0.0f;
-  for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x)
-    s += __ldg(rec + 3 * i).w;
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if ((threadIdx.x & 31) == 0) atomicAdd(out, s);
-}
-
 // dW = sum over the CTAs' partials (column-major blocks, see k_guide_train):
 // 32 weights per block, warp w adds partials w, w + 8, ..., then the eight
 // warp sums are added in warp order (the same order every call).
@@ -774,7 +879,13 @@ __global__ void __launch_bounds__(256) k_dw_reduce(const float* __restrict__ par
   const int e = blockIdx.x * 32 + lane;
   float s = 0.0f;
   if (e < kWSize)
-    for (int c = warp; c < nparts; c += 8) s += __ldg(part + (size_t)c * kWSize + e);
+    for (int c = warp; c < nparts; c += 64) {  // eight loads in flight
+      float v[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[q] = c + 8 * q < nparts ? __ldg(part + (size_t)(c + 8 * q) * kWSize + e) : 0.0f;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) s += v[q];
+    }
   acc[warp][lane] = s;
   __syncthreads();
   if (warp == 0 && e < kWSize) {
@@ -956,7 +1067,7 @@ __global__ void __launch_bounds__(kSampleThreads, kSampleCtasPerSm)
     {
       float u[3], f[16];
       unit_pos(g, f3(q0), u);
-      encode_levels4(g, sres, u, 4 * (int)h, f);
+      encode_levels<4>(g, sres, u, 4 * (int)h, f);
       put8(A, r, 16 * (int)h, f);
       put8(A, r, 16 * (int)h + 8, f + 8);
       if (h == 0) {
@@ -1299,18 +1410,21 @@ void launch_guide_eval(const GuideDev& g, const void* pack, const float* rec, ui
   k_guide_eval<<<(unsigned)grid, kRows, smem, st>>>(g, (const uint4*)pack, (const float4*)rec, n, Y, q, status);
 }
 
-void launch_guide_train(const GuideDev& g, const void* pack, const float* rec, uint64_t n, float* wsum, float* dW,
+void launch_guide_train(const GuideDev& g, const void* pack, const float* rec, uint64_t n, float* scratch, float* dW,
                         float* dWpart, float* dgrid, float* loss, uint32_t* status, int sms, cudaStream_t st) {
-  cudaMemsetAsync(wsum, 0, sizeof(float), st);
-  k_weight_sum<<<sms * 4, 256, 0, st>>>((const float4*)rec, n, wsum);
   const size_t smem = guide_train_smem();
   cudaFuncSetAttribute(k_guide_train, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   const uint64_t tiles = (n + kRows - 1) / kRows;
   uint64_t grid = (uint64_t)sms;
   if (grid > tiles) grid = tiles;
   if (grid == 0) return;
-  k_guide_train<<<(unsigned)grid, kTrainThreads, smem, st>>>(g, (const uint4*)pack, (const float4*)rec, n, wsum, dWpart,
-                                                             dgrid, loss, status);
+  const uint64_t rounds = (n + kTrRound - 1) / kTrRound;
+  const uint64_t chunk = (rounds + kTrMaxChunks - 1) / kTrMaxChunks * kTrRound;
+  const uint32_t nchunks = (uint32_t)((n + chunk - 1) / chunk);
+  uint32_t* ccnt = (uint32_t*)(scratch + kTrMaxChunks);
+  k_guide_count<<<nchunks, 256, 0, st>>>((const float4*)rec, n, chunk, ccnt, scratch, loss);
+  k_guide_train<<<(unsigned)grid, kTrainThreads, smem, st>>>(g, (const uint4*)pack, (const float4*)rec, n, chunk,
+                                                             nchunks, ccnt, scratch, dWpart, dgrid, loss, status);
   k_dw_reduce<<<(kWSize + 31) / 32, 256, 0, st>>>(dWpart, (int)grid, dW);
 }
 
