@@ -83,7 +83,8 @@ typedef struct {
 } rt_camera;
 
 typedef struct {
-  uint32_t wave_capacity;  /* paths in flight per wave; 0 = library default (2^23) */
+  uint32_t wave_capacity;  /* paths in flight per wave; 0 = library default (2^24; 2^23 while paths keep
+                              guide training records or less than 16 GB are free) */
   uint32_t xyz_mode;       /* rt_xyz_mode */
   uint32_t trace_block;    /* threads per block of the traversal kernels, a multiple of 32 up to 128;
                             * 0 = 128 */

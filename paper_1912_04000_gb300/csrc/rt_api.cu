@@ -198,6 +198,21 @@ rt_status ensure_four_band(rt_ctx* c, uint32_t cap) {
   return RT_OK;
 }
 
+// The default wave, where the caller sets none: kSmallWave paths, or kMaxWave
+// where that makes fewer waves and the buffers (120 bytes per path, 180 guided
+// or with four bands) are there already or the device has kWaveRoom free.
+// Every launch of a wave ends with a tail of its longest rays, about 16 us
+// for closest hits and sun rays each: 1024 x 768 x 81 bands x 2 samples of the
+// nave 187.3 ms with 2^23 paths, 183.1 with 2^24; two guided views of the
+// 2M-triangle nave 159.6 and 151.6.
+constexpr uint32_t kSmallWave = 1u << 23;
+constexpr size_t kWaveRoom = (size_t)16 << 30;
+bool wave_room(const rt_ctx* c, uint32_t cap, bool guided, uint32_t nb) {
+  if (c->wave_alloc >= cap && (!guided || c->guide.gq_cap >= cap) && (nb != 4 || c->four_band_alloc >= cap)) return true;
+  size_t free_bytes = 0, all = 0;
+  return cudaMemGetInfo(&free_bytes, &all) == cudaSuccess && free_bytes >= kWaveRoom;
+}
+
 DevScene dev_scene(const rt_ctx* c) {
   DevScene S;
   S.nodes = c->d_nodes;
@@ -973,12 +988,19 @@ static rt_status render_impl(rt_ctx* c, const rt_camera* cams, uint32_t n_cams, 
   cudaSetDevice(c->device);
   cudaStream_t st = c->stream;
   const uint32_t PB = (uint32_t)PB64;
-  uint32_t cap = o.wave_capacity ? o.wave_capacity : (1u << 23);
-  cap = std::max<uint32_t>(std::min<uint32_t>(cap, kMaxWave), 1u);
   // several whole samples per wave where they fit; not where paths keep
   // training slots, whose waves are the batches the guide is trained on
-  const uint32_t m_samples = o.guided && o.guide_collect ? 1u : wave_samples(cap, PB, spp);
-  cap = m_samples > 1 ? m_samples * PB : std::min<uint32_t>(cap, PB);
+  const bool training = o.guided && o.guide_collect;
+  auto wave_cap = [&](uint32_t limit) {
+    const uint32_t m = training ? 1u : wave_samples(limit, PB, spp);
+    return m > 1 ? m * PB : std::min<uint32_t>(limit, PB);
+  };
+  uint32_t cap = wave_cap(o.wave_capacity ? std::min<uint32_t>(o.wave_capacity, kMaxWave) : kSmallWave);
+  if (!o.wave_capacity && !training) {
+    const uint32_t big = wave_cap(kMaxWave);
+    if (big > cap && wave_room(c, big, o.guided, nb)) cap = big;
+  }
+  const uint32_t m_samples = std::max<uint32_t>(1u, cap / PB);
   if (rt_status e = ensure_wave(c, cap)) return e;
   if (nb == 4)
     if (rt_status e = ensure_four_band(c, cap)) return e;
@@ -2004,14 +2026,19 @@ rt_status rt_render_photons(rt_ctx* c, const rt_camera* cams, uint32_t n_cams, u
   const Probe probe{o.probe_map_dev, o.probe_L_dev, o.probe_sig_dev};
   // (whole samples per wave where several fit, as in rt_render; the last
   // chunk's bands may be fewer and its samples smaller)
-  constexpr uint64_t kPhotonWave = 1u << 23;
-  static_assert(kPhotonWave <= kMaxWave, "wave capacity");
+  uint64_t wave_limit = kSmallWave;
   const uint32_t bc_last = band_count % Bc ? band_count % Bc : Bc;
   auto wave_of = [&](uint64_t bc) {
     const uint64_t pb = npix * bc;
-    return std::max<uint64_t>(1, std::min(kPhotonWave, pb * wave_samples(kPhotonWave, pb, spp)));
+    return std::max<uint64_t>(1, std::min(wave_limit, pb * wave_samples(wave_limit, pb, spp)));
   };
-  const uint32_t cap = (uint32_t)std::max(wave_of(Bc), wave_of(bc_last));
+  uint32_t cap = (uint32_t)std::max(wave_of(Bc), wave_of(bc_last));
+  wave_limit = kMaxWave;
+  const uint32_t big = (uint32_t)std::max(wave_of(Bc), wave_of(bc_last));
+  if (big > cap && wave_room(c, big, false, 1u))
+    cap = big;
+  else
+    wave_limit = kSmallWave;
   if (rt_status e = ensure_wave(c, cap)) return e;
   LaunchCfg lc;
   lc.block_trace = 128;
