@@ -996,7 +996,8 @@ static rt_status render_impl(rt_ctx* c, const rt_camera* cams, uint32_t n_cams, 
     return m > 1 ? m * PB : std::min<uint32_t>(limit, PB);
   };
   uint32_t cap = wave_cap(o.wave_capacity ? std::min<uint32_t>(o.wave_capacity, kMaxWave) : kSmallWave);
-  if (!o.wave_capacity && !training) {
+  // (in-sample indices of a wave stay below 2^32)
+  if (!o.wave_capacity && !training && PB64 + kMaxWave < (1ull << 32)) {
     const uint32_t big = wave_cap(kMaxWave);
     if (big > cap && wave_room(c, big, o.guided, nb)) cap = big;
   }
@@ -2035,7 +2036,7 @@ rt_status rt_render_photons(rt_ctx* c, const rt_camera* cams, uint32_t n_cams, u
   uint32_t cap = (uint32_t)std::max(wave_of(Bc), wave_of(bc_last));
   wave_limit = kMaxWave;
   const uint32_t big = (uint32_t)std::max(wave_of(Bc), wave_of(bc_last));
-  if (big > cap && wave_room(c, big, false, 1u))
+  if (big > cap && npix * Bc + kMaxWave < (1ull << 32) && wave_room(c, big, false, 1u))
     cap = big;
   else
     wave_limit = kSmallWave;

@@ -973,13 +973,8 @@ __global__ void __launch_bounds__(256) k_camera(const DevCam* __restrict__ cams,
 }
 
 constexpr uint32_t kNoRay = 0xFFFFFFFFu;
-// closest-hit kernel: blocks of at most 128 threads, launch bound 8 blocks
-// per SM (<= 64 registers; the closest-hit kernel compiles to 56 and the
-// launch takes the occupancy limit, 9 blocks, the one-band sun-ray kernel to
-// 61 and 8 blocks).  With the 256-bit node loads, measured per render of the
-// nave / the 2M-triangle nave, closest hit: bound 8 1372 / 2141 ms, bound 9
-// 1384 / 2160, 7 and 6 about 1408 / 2200, 10 and 12 (spilled) 27% and 40%
-// slower: more warps thrash the L1 that serves the node fetches
+// The kernels over the other trees (trace_variant 1 to 5): blocks of at most
+// 128 threads, launch bound 8 blocks per SM (<= 64 registers, none spilled).
 #ifndef SRT_TRACE_MIN_BLOCKS
 #define SRT_TRACE_MIN_BLOCKS 8
 #endif
@@ -1291,6 +1286,9 @@ struct BlockAppend {
 // 34.8 / 23.1; 6 blocks of 128 31.8 / 21.1, 7 29.3 / 19.7, 8 28.7 / 19.4 (64
 // registers), 9 28.7 / 18.9, 10 29.8 / 20.0.  Four bands (512 x 384 crystal nave, 4
 // samples): 13.2 ms, then 11.5 with 3 blocks of 256, 10.3 with 4, 10.8 with 8 of 128.
+// With the path's radiance touched only at vertices that add to it (waves of
+// 2^24 paths): 29.0 / 19.0 -> 26.7 / 17.6 ms, four bands 10.6 -> 10.0; copying
+// the next turn's ray and hit ahead (cp.async) gave half of that back.
 constexpr int kShadeThreads = 128, kShadeBlocksPerSm = 8;
 constexpr int kShade4Threads = 256, kShade4BlocksPerSm = 4;
 template <bool RECORD, bool GUIDED, bool PM = false>
@@ -1320,18 +1318,20 @@ __global__ void __launch_bounds__(kShadeThreads, kShadeBlocksPerSm) k_shade(DevS
       const float3 o = f3(a), d = f3(b);
       const PathId id = path_id(w, pid);
       const uint32_t band = w.band_first + id.j;
-      float Lp = Lbuf[pid];
+      // the path's radiance is read and written only where this vertex adds to
+      // it or ends the path
+      auto add_light = [&](float x, float y) { Lbuf[pid] = fmaf(x, y, Lbuf[pid]); };
       uint32_t sg = RECORD ? sigbuf[pid] : 0u;
       // training slot of the previous (guided) vertex: radiance gathered so far
       if (GUIDED && gw.collect != 0u && k >= 2u && k - 1u <= gw.depth && pid % gw.collect == 0u)
-        ((float*)(gw.raw + kRawF4 * ((k - 2u) * gw.slots_per_vertex + pid / gw.collect) + 1u))[3] = Lp;
+        ((float*)(gw.raw + kRawF4 * ((k - 2u) * gw.slots_per_vertex + pid / gw.collect) + 1u))[3] = Lbuf[pid];
       const int leaf = __float_as_int(h.y);
       bool terminate = false;
       if (leaf < 0) {
         if (RECORD) sg = mix_sig(sg, 0xFFFFFFFFu);
         if (dot(d, P.sun) >= P.cos_max) {
-          if (!covered) Lp += T * __ldg(P.sunL + band);
-          else if (GUIDED && (bits & kFlagGuidedEsc)) Lp += T * __ldg(P.sunL + band) * gw.wesc[pid];
+          if (!covered) add_light(T, __ldg(P.sunL + band));
+          else if (GUIDED && (bits & kFlagGuidedEsc)) add_light(T * __ldg(P.sunL + band), gw.wesc[pid]);
         }
         terminate = true;
       } else {
@@ -1346,7 +1346,7 @@ __global__ void __launch_bounds__(kShadeThreads, kShadeBlocksPerSm) k_shade(DevS
         const int type = __ldg(P.mtype + mat);
         const uint4 u = philox4x32_10(make_uint4(id.pix, id.s, band, 4u * k), w.key0, w.key1);
         if (type == 0 || type == 3) {
-          if (type == 3) Lp += T * m.w;
+          if (type == 3) add_light(T, m.w);
           // next-event estimate: uniform direction in the sun cone
           const float om = u01(u.x) * P.one_minus_cos;
           const float ct = 1.0f - om;
@@ -1368,7 +1368,7 @@ __global__ void __launch_bounds__(kShadeThreads, kShadeBlocksPerSm) k_shade(DevS
           }
           if (PM) {
             const float E = photon_gather(pm, 0u, id.j, p) * pm.norm[0] + photon_gather(pm, 1u, id.j, p) * pm.norm[1];
-            Lp += T * m.z * (1.0f / 3.14159265358979f) * E;
+            add_light(T * m.z * (1.0f / 3.14159265358979f), E);
             terminate = true;
           } else if (k == w.depth) {
             terminate = true;
@@ -1461,11 +1461,11 @@ __global__ void __launch_bounds__(kShadeThreads, kShadeBlocksPerSm) k_shade(DevS
         }
       }
       if (terminate && !emit_shadow) {
+        const float Lp = Lbuf[pid];
         finalize(w, id, pid, Lp, sg, Lbuf, accum, probe, RECORD);
         if (GUIDED && gw.Lfinal) gw.Lfinal[pid] = Lp;
-      } else {
-        Lbuf[pid] = Lp;
-        if (RECORD) sigbuf[pid] = sg;
+      } else if (RECORD) {
+        sigbuf[pid] = sg;
       }
     }
     const bool want[3] = {emit_next, emit_shadow, emit_guide};
@@ -1550,17 +1550,23 @@ __global__ void __launch_bounds__(kShade4Threads, kShade4BlocksPerSm) k_shade4(D
       const PathId id = path_id(w, pid);
       const uint32_t b0 = w.band_first + id.j, G = w.band_count;
       const uint32_t nv = four_band_count(w, id.j);
-      const float4 t4 = T4[pid], l4 = L4[pid];
-      float T[4] = {t4.x, t4.y, t4.z, t4.w}, L[4] = {l4.x, l4.y, l4.z, l4.w};
+      const float4 t4 = T4[pid];
+      float T[4] = {t4.x, t4.y, t4.z, t4.w};
+      // as in k_shade, the radiances are touched only where they change
+      auto add_light = [&](const float (&le)[4]) {
+        const float4 l = L4[pid];
+        L4[pid] = make_float4(fmaf(T[0], le[0], l.x), fmaf(T[1], le[1], l.y), fmaf(T[2], le[2], l.z), fmaf(T[3], le[3], l.w));
+      };
       uint32_t sg = RECORD ? sigbuf[pid] : 0u;
       const int leaf = __float_as_int(h.y);
       bool terminate = false;
       if (leaf < 0) {
         if (RECORD) sg = mix_sig(sg, 0xFFFFFFFFu);
         if (!covered && dot(d, P.sun) >= P.cos_max) {
+          float le[4];
 #pragma unroll
-          for (uint32_t q = 0; q < 4u; ++q)
-            if (q < nv) L[q] += T[q] * __ldg(P.sunL + b0 + q * G);
+          for (uint32_t q = 0; q < 4u; ++q) le[q] = q < nv ? __ldg(P.sunL + b0 + q * G) : 0.0f;
+          add_light(le);
         }
         terminate = true;
       } else {
@@ -1589,9 +1595,10 @@ __global__ void __launch_bounds__(kShade4Threads, kShade4BlocksPerSm) k_shade4(D
 #pragma unroll
           for (uint32_t q = 0; q < 4u; ++q) rho[q] = q < nv ? __ldg(&mr[q * G].z) : 0.0f;
           if (type == 3) {
+            float le[4];
 #pragma unroll
-            for (uint32_t q = 0; q < 4u; ++q)
-              if (q < nv) L[q] += T[q] * __ldg(&mr[q * G].w);
+            for (uint32_t q = 0; q < 4u; ++q) le[q] = q < nv ? __ldg(&mr[q * G].w) : 0.0f;
+            add_light(le);
           }
           const float om = u01(u.x) * P.one_minus_cos;
           const float ct = 1.0f - om;
@@ -1763,10 +1770,11 @@ __global__ void __launch_bounds__(kShade4Threads, kShade4BlocksPerSm) k_shade4(D
         }
       }
       if (terminate && !emit_shadow) {
+        const float4 l4 = L4[pid];
+        const float L[4] = {l4.x, l4.y, l4.z, l4.w};
         finalize4(w, id, pid, L, sg, L4, accum, probe, RECORD);
-      } else {
-        L4[pid] = make_float4(L[0], L[1], L[2], L[3]);
-        if (RECORD) sigbuf[pid] = sg;
+      } else if (RECORD) {
+        sigbuf[pid] = sg;
       }
       if (emit_next) T4[pid] = make_float4(T[0], T[1], T[2], T[3]);
     }
@@ -1803,8 +1811,11 @@ __device__ __forceinline__ void sun_ray_done(const DevSpectra& P, const WavePara
                                              float* __restrict__ Lbuf, uint32_t* __restrict__ sigbuf,
                                              double* __restrict__ accum, const Probe& probe, float* Lfinal) {
   const uint32_t pid = bits & kPidMask;
+  // an occluded ray that neither ends its path nor leaves a record changes
+  // nothing (sun rays of the 1024 x 768 nave 33.6 -> 32.9 ms, four bands 5.33 -> 5.18)
+  if (!RECORD && !rec_sun && !(bits & kFlagTerm) && contrib * T == 0.0f) return;
   const PathId id = path_id(w, pid);
-  const float Lp = Lbuf[pid] + contrib * T;
+  const float Lp = fmaf(contrib, T, Lbuf[pid]);
   if (rec_sun && pid % gw.collect == 0u)
     ((float*)(gw.raw + kRawF4 * ((k - 1u) * gw.slots_per_vertex + pid / gw.collect) + 5u))[0] =
         T * __ldg(P.sunL + w.band_first + id.j);
@@ -1826,8 +1837,9 @@ __device__ __forceinline__ void sun_ray_done4(const WaveParams& w, uint32_t bits
                                               uint32_t* __restrict__ sigbuf, double* __restrict__ accum,
                                               const Probe& probe) {
   const uint32_t pid = bits & kPidMask;
+  if (!RECORD && !(bits & kFlagTerm) && T[0] == 0.0f && T[1] == 0.0f && T[2] == 0.0f && T[3] == 0.0f) return;
   const float4 c4 = C4[pid], l4 = L4[pid];
-  const float L[4] = {l4.x + c4.x * T[0], l4.y + c4.y * T[1], l4.z + c4.z * T[2], l4.w + c4.w * T[3]};
+  const float L[4] = {fmaf(c4.x, T[0], l4.x), fmaf(c4.y, T[1], l4.y), fmaf(c4.z, T[2], l4.z), fmaf(c4.w, T[3], l4.w)};
   uint32_t sg = 0;
   if (RECORD) sg = mix_sig(sigbuf[pid], ng);
   if (bits & kFlagTerm) {
@@ -2437,7 +2449,7 @@ void launch_wave(const LaunchCfg& lcfg, const DevScene& S, const DevSpectra& P, 
     }
     // vertex 1 starts at the cameras: where one lies outside the scene bounds,
     // the box test for any origin; later origins are surface points inside the
-    // padded bounds (all closest hits of 1280 x 960 x 81 bands x 4 samples in
+    // padded bounds (all closest hits of 1024 x 768 x 81 bands x 2 samples in
     // the 98k-triangle nave: 122.2 ms, with the general test at vertex 1 124.6)
     launch_trace(lc, k == 1 && !lc.cams_inside, S, qin, b, k, st);
     if (tm) tm->end(STG_TRACE, st);
