@@ -691,7 +691,7 @@ def main():
                 "paths_per_step_per_gpu": P * B, "accumulation": "f64",
                 "guide": f"8-lobe vMF MLP guide, one-sample MIS alpha 0.7, guide depth 2, trained online in every "
                          f"pass (every {GUIDE_COLLECT}th path, {GUIDE_STEPS} Adam steps per wave)",
-                "xyz": "bf16x3 tensor cores, f32 accumulate",
+                "xyz": "f32",
                 "l2": "inputs larger than L2: 2M-triangle BVH and triangles (about 0.3 GB), 1.1 GB of wave queues "
                       "and an 8.2 GB FP64 spectral image per step",
                 "partition": ("each rank renders its band sub-domain of every pass; XYZ partials reduced to rank 0 "
