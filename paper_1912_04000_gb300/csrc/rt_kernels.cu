@@ -35,9 +35,18 @@ namespace {
 // FMA selects the box test: false = (plane - o) * inv (any origin); true =
 // fma(plane, inv, -o * inv), valid for origins within the scene bounds
 // because rt_load_scene pads every node box by 2^-22 (max |coordinate| + eps),
-// which covers the rounding of o * inv; the far distance is widened by
-// 1 + 2^-21 for the relative rounding of both distances.
+// which covers the rounding of o * inv; the entry distance is shortened by
+// kNearMargin for the relative rounding of both distances.
 // ---------------------------------------------------------------------------
+// Entry distances are shortened by 2^-21 (8 of u = 2^-24) before they are
+// compared with exit and hit distances, at the box test and, as the stacks
+// hold them shortened, when an entry is popped: of an entry distance t the
+// padding leaves up to 4 u t uncovered (2 by the four-wide kernels' approximate
+// reciprocal, 1 by each rounding after it), the other 4 u t are the hit's.
+// Entries popped by the unshortened distance dropped boxes that held a hit at
+// an equal or rounding-nearer distance.
+constexpr float kNearMargin = 1.0f - 0x1p-21f;
+
 struct Trav {
   RayW rw;
   float3 inv, oinv;
@@ -69,9 +78,9 @@ __device__ __forceinline__ float box_t(const Trav& tv, float4 lo, float4 hi, flo
     tz0 = __fmul_rn(__fsub_rn(lo.z, tv.oinv.z), tv.inv.z);
     tz1 = __fmul_rn(__fsub_rn(hi.z, tv.oinv.z), tv.inv.z);
   }
-  const float tn = fmaxf(fmaxf(fminf(tx0, tx1), fminf(ty0, ty1)), fmaxf(fminf(tz0, tz1), 0.0f));
+  const float tn = kNearMargin * fmaxf(fmaxf(fminf(tx0, tx1), fminf(ty0, ty1)), fmaxf(fminf(tz0, tz1), 0.0f));
   const float tf = fminf(fminf(fmaxf(tx0, tx1), fmaxf(ty0, ty1)), fminf(fmaxf(tz0, tz1), tmax));
-  return (tn <= tf * 1.0000005f) ? tn : -1.0f;
+  return tn <= tf ? tn : -1.0f;
 }
 
 // Starts a ray; returns false if it misses the root box (finished).
@@ -222,7 +231,7 @@ __device__ __forceinline__ float min3f(float a, float b, float c) {
 }
 
 // The reciprocals only bound boxes: their 1 ulp error scales both distances
-// of a slab alike and is covered by the far distance's margin.
+// of a slab alike and is covered by kNearMargin.
 template <bool FMA>
 __device__ __forceinline__ void ray4_init(Ray4& r, const RayRows& rows, float3 o, float3 d) {
   rows.put(ray_prep(o, d));
@@ -270,9 +279,9 @@ __device__ __forceinline__ float child4(const Ray4& r, float cx, float hx, float
   slab4<FMA>(cx, hx, r.inv.x, r.ainv.x, r.oinv.x, nx, fx);
   slab4<FMA>(cy, hy, r.inv.y, r.ainv.y, r.oinv.y, ny, fy);
   slab4<FMA>(cz, hz, r.inv.z, r.ainv.z, r.oinv.z, nz, fz);
-  const float tn = max3f(nx, ny, fmaxf(nz, 0.0f));
+  const float tn = kNearMargin * max3f(nx, ny, fmaxf(nz, 0.0f));
   const float tf = min3f(fx, fy, fminf(fz, tmax));
-  return tn <= tf * 1.0000005f ? tn : INFINITY;
+  return tn <= tf ? tn : INFINITY;
 }
 
 __device__ __forceinline__ void cswap(float& ta, uint32_t& pa, float& tb, uint32_t& pb) {
@@ -431,11 +440,11 @@ __device__ __forceinline__ float slab(float plane, float inv, float oinv) {
 template <bool FMA>
 __device__ __forceinline__ float child_t(const Trav& tv, float nx, float fx, float ny, float fy, float nz, float fz,
                                          float tmax) {
-  const float tn = fmaxf(fmaxf(slab<FMA>(nx, tv.inv.x, tv.oinv.x), slab<FMA>(ny, tv.inv.y, tv.oinv.y)),
-                         fmaxf(slab<FMA>(nz, tv.inv.z, tv.oinv.z), 0.0f));
+  const float tn = kNearMargin * fmaxf(fmaxf(slab<FMA>(nx, tv.inv.x, tv.oinv.x), slab<FMA>(ny, tv.inv.y, tv.oinv.y)),
+                                       fmaxf(slab<FMA>(nz, tv.inv.z, tv.oinv.z), 0.0f));
   const float tf = fminf(fminf(slab<FMA>(fx, tv.inv.x, tv.oinv.x), slab<FMA>(fy, tv.inv.y, tv.oinv.y)),
                          fminf(slab<FMA>(fz, tv.inv.z, tv.oinv.z), tmax));
-  return tn <= tf * 1.0000005f ? tn : INFINITY;
+  return tn <= tf ? tn : INFINITY;
 }
 
 template <bool FMA>
@@ -503,11 +512,11 @@ __device__ __forceinline__ bool trav_interior4q(Trav& tv, uint2* stack, const De
 #pragma unroll
   for (uint32_t i = 0; i < 4; ++i) {
     const uint32_t sel = 0x7540u | i;
-    const float tn = fmaxf(fmaxf(fmaf(qplane(nx, sel), sx, bx), fmaf(qplane(ny, sel), sy, by)),
-                           fmaxf(fmaf(qplane(nz, sel), sz, bz), 0.0f));
+    const float tn = kNearMargin * fmaxf(fmaxf(fmaf(qplane(nx, sel), sx, bx), fmaf(qplane(ny, sel), sy, by)),
+                                         fmaxf(fmaf(qplane(nz, sel), sz, bz), 0.0f));
     const float tf = fminf(fminf(fmaf(qplane(fx, sel), sx, bx), fmaf(qplane(fy, sel), sy, by)),
                            fminf(fmaf(qplane(fz, sel), sz, bz), tmax));
-    t[i] = tn <= tf * 1.0000005f ? tn : INFINITY;
+    t[i] = tn <= tf ? tn : INFINITY;
   }
   float t0 = t[0], t1 = t[1], t2 = t[2], t3 = t[3];
   uint32_t p0 = pk.x, p1 = pk.y, p2 = pk.z, p3 = pk.w;
