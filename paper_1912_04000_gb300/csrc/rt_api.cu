@@ -155,9 +155,19 @@ rt_status check_ctx(rt_ctx* c) {
   return RT_OK;
 }
 
+// Forgets the captured render: it holds the addresses of the buffers it was
+// captured with, of which its key names only some.  Called wherever one of
+// them is freed.
+void drop_graph(rt_ctx* c) {
+  if (c->graph_exec) cudaGraphExecDestroy(c->graph_exec);
+  c->graph_exec = nullptr;
+  c->graph_key.clear();
+}
+
 rt_status ensure_wave(rt_ctx* c, uint32_t cap) {
   if (c->wave_alloc >= cap) return RT_OK;
   WaveBufs& b = c->wb;
+  drop_graph(c);
   dfree(b.q[0]);
   dfree(b.q[1]);
   dfree(b.hit);
@@ -187,6 +197,7 @@ rt_status ensure_wave(rt_ctx* c, uint32_t cap) {
 rt_status ensure_four_band(rt_ctx* c, uint32_t cap) {
   if (c->four_band_alloc >= cap) return RT_OK;
   WaveBufs& b = c->wb;
+  drop_graph(c);
   dfree(b.L4);
   dfree(b.T4);
   dfree(b.C4);
@@ -413,7 +424,7 @@ void rt_destroy(rt_ctx* c) {
   for (auto& e : c->ev)
     if (e) cudaEventDestroy(e);
   for (auto& e : c->tpool) cudaEventDestroy(e);
-  if (c->graph_exec) cudaGraphExecDestroy(c->graph_exec);
+  drop_graph(c);
   if (c->gstream) cudaStreamDestroy(c->gstream);
   delete c;
 }
@@ -437,7 +448,7 @@ rt_status rt_set_limits(rt_ctx* c, uint32_t queue_capacity, uint32_t traversal_s
   c->lim_queue = queue_capacity;
   c->lim_steps = traversal_steps;
   c->fail_countdown = fail_cuda_call;
-  c->graph_key.clear();  // a captured render holds the old limits
+  drop_graph(c);  // a captured render holds the old limits
   return RT_OK;
 }
 
@@ -1010,6 +1021,7 @@ static rt_status render_impl(rt_ctx* c, const rt_camera* cams, uint32_t n_cams, 
   double* accum = spectral_dev;
   if (!accum) {
     if (c->accum_cap < ACC64) {
+      drop_graph(c);
       dfree(c->d_accum);
       c->accum_cap = 0;
       CUDA_TRY(c, cudaMalloc(&c->d_accum, ACC64 * sizeof(double)));
@@ -1063,6 +1075,7 @@ static rt_status render_impl(rt_ctx* c, const rt_camera* cams, uint32_t n_cams, 
     gw.depth = std::min<uint32_t>(G.cfg.guide_depth, depth);
     gw.alpha = G.cfg.mis_alpha;
     if (G.gq_cap < cap) {
+      drop_graph(c);
       dfree(G.gq);
       dfree(G.wesc);
       dfree(G.perm);
@@ -1088,6 +1101,7 @@ static rt_status render_impl(rt_ctx* c, const rt_camera* cams, uint32_t n_cams, 
       gw.slots_per_vertex = (cap + o.guide_collect - 1) / o.guide_collect;
       n_slots = gw.slots_per_vertex * gw.depth;
       if (G.raw_cap < n_slots || !G.Lfinal) {
+        drop_graph(c);
         dfree(G.raw);
         dfree(G.trec);
         dfree(G.Lfinal);
@@ -1213,10 +1227,7 @@ static rt_status render_impl(rt_ctx* c, const rt_camera* cams, uint32_t n_cams, 
     for (uint32_t v = 0; v < n_cams; ++v) key += "|" + std::to_string(cams[v].width) + "x" + std::to_string(cams[v].height);
     if (!c->gstream) CUDA_TRY(c, cudaStreamCreateWithFlags(&c->gstream, cudaStreamNonBlocking));
     if (!c->graph_exec || key != c->graph_key) {
-      if (c->graph_exec) {
-        cudaGraphExecDestroy(c->graph_exec);
-        c->graph_exec = nullptr;
-      }
+      drop_graph(c);
       CUDA_TRY(c, cudaStreamBeginCapture(c->gstream, cudaStreamCaptureModeThreadLocal));
       const cudaError_t ce = enqueue(c->gstream, false);
       cudaGraph_t g = nullptr;
@@ -1279,6 +1290,7 @@ rt_status rt_render_host(rt_ctx* c, const rt_camera* cams, uint32_t n_cams, uint
   for (uint32_t v = 0; v < n_cams; ++v) npix += (uint64_t)cams[v].width * cams[v].height;
   cudaSetDevice(c->device);
   if (c->xyz_cap < npix * 3) {
+    drop_graph(c);
     dfree(c->d_xyz);
     c->xyz_cap = 0;
     CUDA_TRY(c, cudaMalloc(&c->d_xyz, npix * 3 * sizeof(float)));
@@ -1987,6 +1999,7 @@ rt_status rt_render_photons(rt_ctx* c, const rt_camera* cams, uint32_t n_cams, u
   double* accum = spectral_dev;
   if (!accum) {
     if (c->accum_cap < ACC64) {
+      drop_graph(c);
       dfree(c->d_accum);
       c->accum_cap = 0;
       CUDA_TRY(c, cudaMalloc(&c->d_accum, ACC64 * sizeof(double)));
