@@ -156,8 +156,9 @@ rt_status check_ctx(rt_ctx* c) {
 }
 
 // Forgets the captured render: it holds the addresses of the buffers it was
-// captured with, of which its key names only some.  Called wherever one of
-// them is freed.
+// captured with, of which its key names only some, and by value the scene's
+// bounds and counts, the sun and the guide's grid resolutions.  Called wherever
+// one of them is freed or set.
 void drop_graph(rt_ctx* c) {
   if (c->graph_exec) cudaGraphExecDestroy(c->graph_exec);
   c->graph_exec = nullptr;
@@ -705,6 +706,7 @@ rt_status rt_load_scene(rt_ctx* c, const float* verts, uint32_t n_verts, const u
   }
   cudaSetDevice(c->device);
   if (c->stream) cudaStreamSynchronize(c->stream);
+  drop_graph(c);
   dfree(c->d_nodes);
   dfree(c->d_nodes4);
   dfree(c->d_nodes8);
@@ -836,6 +838,7 @@ rt_status rt_set_spectra(rt_ctx* c, const float* lambda_nm, uint32_t n_bands, co
     }
   cudaSetDevice(c->device);
   if (c->stream) cudaStreamSynchronize(c->stream);
+  drop_graph(c);
   dfree(c->d_mb);
   dfree(c->d_ad);
   dfree(c->d_mtype);
@@ -1419,6 +1422,7 @@ rt_status rt_guide_init(rt_ctx* c, const rt_guide_config* cfg_in, uint64_t seed)
     return fail(c, RT_ERR_ARG, "rt_guide_init: bad configuration");
   auto& G = c->guide;
   cudaSetDevice(c->device);
+  drop_graph(c);
   const uint64_t T = 1ull << cfg.log2_table;
   const uint64_t ng = (uint64_t)kGuideLevels * T * kGuideFeatures;
   if (G.n_grid != ng) {
