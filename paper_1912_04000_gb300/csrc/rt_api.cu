@@ -211,8 +211,11 @@ rt_status ensure_four_band(rt_ctx* c, uint32_t cap) {
 }
 
 // The default wave, where the caller sets none: kSmallWave paths, or kMaxWave
-// where that makes fewer waves and the buffers (120 bytes per path, 180 guided
-// or with four bands) are there already or the device has kWaveRoom free.
+// where that makes fewer waves and the buffers are there already or the device
+// has kWaveRoom free: kMaxWave paths take 2 GB (120 bytes each; 3 GB guided or
+// with four bands, 180 each), a fifth of it at most.  Asked when all else that
+// the render holds is allocated: an image that leaves less than this room is
+// rendered in small waves.
 // Every launch of a wave ends with a tail of its longest rays, about 16 us
 // for closest hits and sun rays each: 1024 x 768 x 81 bands x 2 samples of the
 // nave 187.3 ms with 2^23 paths, 183.1 with 2^24; two guided views of the
@@ -1002,6 +1005,19 @@ static rt_status render_impl(rt_ctx* c, const rt_camera* cams, uint32_t n_cams, 
   cudaSetDevice(c->device);
   cudaStream_t st = c->stream;
   const uint32_t PB = (uint32_t)PB64;
+  if (spectral_dev && ((uintptr_t)spectral_dev & 15u) != 0)
+    return fail(c, RT_ERR_ARG, "rt_render: spectral_dev must be 16-byte aligned");
+  double* accum = spectral_dev;
+  if (!accum) {
+    if (c->accum_cap < ACC64) {
+      drop_graph(c);
+      dfree(c->d_accum);
+      c->accum_cap = 0;
+      CUDA_TRY(c, cudaMalloc(&c->d_accum, ACC64 * sizeof(double)));
+      c->accum_cap = ACC64;
+    }
+    accum = c->d_accum;
+  }
   // several whole samples per wave where they fit; not where paths keep
   // training slots, whose waves are the batches the guide is trained on
   const bool training = o.guided && o.guide_collect;
@@ -1019,19 +1035,6 @@ static rt_status render_impl(rt_ctx* c, const rt_camera* cams, uint32_t n_cams, 
   if (rt_status e = ensure_wave(c, cap)) return e;
   if (nb == 4)
     if (rt_status e = ensure_four_band(c, cap)) return e;
-  if (spectral_dev && ((uintptr_t)spectral_dev & 15u) != 0)
-    return fail(c, RT_ERR_ARG, "rt_render: spectral_dev must be 16-byte aligned");
-  double* accum = spectral_dev;
-  if (!accum) {
-    if (c->accum_cap < ACC64) {
-      drop_graph(c);
-      dfree(c->d_accum);
-      c->accum_cap = 0;
-      CUDA_TRY(c, cudaMalloc(&c->d_accum, ACC64 * sizeof(double)));
-      c->accum_cap = ACC64;
-    }
-    accum = c->d_accum;
-  }
   if (o.trace_block && (o.trace_block > 128 || o.trace_block % 32))
     return fail(c, RT_ERR_ARG, "rt_render: trace_block must be a multiple of 32 up to 128");
   LaunchCfg lc;
