@@ -88,9 +88,10 @@ __device__ __forceinline__ float f64_to_f32_rz(uint32_t lo, uint32_t hi) {
 
 // FP64 -> FP32, nearest (ties away from zero): one bit more than the 23 kept,
 // plus one, halved.  Magnitudes below the FP32 normal range give signed zero.
-// top keeps the largest rebiased high word: past kTopF32 a value lies above
-// the FP32 range or is not finite, and its result is wrong.
-constexpr int kTopF32 = (1150 - 896) << 20;
+// top keeps the largest rebiased high word: past kTopF32 a value is above
+// 2^96, where 192 products with weights of up to 2^24 can leave the FP32 range
+// before the division by the samples (and the value itself can).
+constexpr int kTopF32 = (1023 + 96 - 896) << 20;
 __device__ __forceinline__ float f64_to_f32_rn(uint2 d, int& top) {
   const int t = (int)((d.y & 0x7FFFFFFFu) - (896u << 20));
   top = max(top, t);
@@ -395,9 +396,10 @@ size_t xyz_f32_smem(uint32_t bc) {
 template <int RPT>
 __global__ void __launch_bounds__(kF32Threads, 2)
     k_xyz_f32(const double* __restrict__ s, uint64_t np, uint32_t bc, uint32_t n_stages, const float* __restrict__ w,
-              float inv_spp, float* __restrict__ xyz, uint32_t* status) {
+              double inv_spp, float* __restrict__ xyz, uint32_t* status) {
   extern __shared__ __align__(1024) unsigned char smem[];
   constexpr uint32_t kRows = 32u * RPT;
+  const float inv_spp_f = (float)inv_spp;
   const uint32_t stage_bytes = kRows * bc * 8u;  // a multiple of 256
   float4* W = (float4*)(smem + n_stages * stage_bytes);
   uint64_t* full = (uint64_t*)(W + bc);
@@ -458,14 +460,18 @@ __global__ void __launch_bounds__(kF32Threads, 2)
         z[q] = fmaf(f, c.z, z[q]);
       }
     }
-    if (top > kTopF32) {  // a sum above the FP32 range, an infinity or a NaN: by the conversion instruction
+    // a large value, an infinity or a NaN in the warp's pixels: divided in FP64
+    // before the conversion, by its instruction
+    float scale = inv_spp_f;
+    if (__any_sync(0xffffffffu, top > kTopF32)) {
+      scale = 1.0f;
 #pragma unroll
       for (int q = 0; q < RPT; ++q) {
         x[q] = y[q] = z[q] = 0.0f;
         for (uint32_t j = l; j < bc; j += 8u) {
           const float4 c = W[j];
           const uint2 d = v[q][j];
-          const float f = (float)__hiloint2double((int)d.y, (int)d.x);
+          const float f = (float)(__hiloint2double((int)d.y, (int)d.x) * inv_spp);
           x[q] = fmaf(f, c.x, x[q]);
           y[q] = fmaf(f, c.y, y[q]);
           z[q] = fmaf(f, c.z, z[q]);
@@ -481,7 +487,7 @@ __global__ void __launch_bounds__(kF32Threads, 2)
         z[q] += __shfl_xor_sync(0xffffffffu, z[q], o);
       }
       const uint64_t p = p0 + 32u * (uint32_t)q;
-      if (p < np && l < 3u) xyz[3 * p + l] = (l == 0 ? x[q] : (l == 1 ? y[q] : z[q])) * inv_spp;
+      if (p < np && l < 3u) xyz[3 * p + l] = (l == 0 ? x[q] : (l == 1 ? y[q] : z[q])) * scale;
     }
     // the stage is read: refill it
     __syncthreads();
@@ -522,8 +528,7 @@ void launch_xyz(const double* spectral, uint64_t n_pixels, const XyzWeights& w, 
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     const uint64_t nt = (n_pixels + 32 * rpt - 1) / (32 * rpt);
     const unsigned grid = (unsigned)(nt < 2ull * (uint64_t)sms ? nt : 2ull * (uint64_t)sms);
-    kernel<<<grid, kF32Threads, smem, st>>>(spectral, n_pixels, w.band_count, n_stages, w.w32, (float)(1.0 / (double)spp),
-                                          xyz, status);
+    kernel<<<grid, kF32Threads, smem, st>>>(spectral, n_pixels, w.band_count, n_stages, w.w32, 1.0 / (double)spp, xyz, status);
     return;
   }
   const uint32_t nk = (w.band_count + 15) / 16;
