@@ -124,7 +124,8 @@ typedef struct {
   uint32_t sample_first;
   uint32_t accumulate;
   uint32_t spp_total;
-  uint32_t leaf_batch;     /* trace_variant 0: 1..32 waiting lanes start a leaf phase; 0 = default */
+  uint32_t leaf_batch;     /* 1..32 waiting lanes start a leaf phase of closest hits; 0 = default (16).
+                            * Sun rays over the four-wide BVH: 10 more, at most 28 */
   uint32_t guide_order;    /* guided: 0 = guide queries in queue order (the default: measured
                             * faster), 1 = sorted by position first (Morton order of a 64^3 grid,
                             * so that a tile's hash-grid gathers share cache lines); the same bits */

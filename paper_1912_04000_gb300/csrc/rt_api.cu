@@ -1047,7 +1047,7 @@ static rt_status render_impl(rt_ctx* c, const rt_camera* cams, uint32_t n_cams, 
   lc.record = o.probe_map_dev != nullptr;
   lc.variant = (int)o.trace_variant;
   lc.leaf_min = o.leaf_batch ? (int)o.leaf_batch : kDefaultLeafBatch;
-  lc.shadow_leaf = o.leaf_batch ? (int)o.leaf_batch : kDefaultShadowLeafBatch;
+  lc.shadow_leaf = shadow_leaf_batch(lc.leaf_min);
   lc.sort_rays = o.ray_order == 1;
   // (rounds of at most kMaxSteps steps: the kernels check a ray's step limit between rounds)
   constexpr uint32_t kMaxSteps = 1024;
@@ -2071,7 +2071,7 @@ rt_status rt_render_photons(rt_ctx* c, const rt_camera* cams, uint32_t n_cams, u
   lc.record = o.probe_map_dev != nullptr;
   lc.variant = 0;
   lc.leaf_min = kDefaultLeafBatch;
-  lc.shadow_leaf = kDefaultShadowLeafBatch;
+  lc.shadow_leaf = shadow_leaf_batch(lc.leaf_min);
   lc.sort_rays = false;
   lc.trace_steps = kDefaultTraceSteps;
   lc.trace_refill = kDefaultTraceRefill;

@@ -263,7 +263,12 @@ struct Probe {
 constexpr int kDefaultTraceSteps = 8, kDefaultTraceRefill = 8;
 constexpr int kDefaultShadowSteps = 8, kDefaultShadowRefill = 12;
 constexpr int kDefaultLeafBatch = 16;
-constexpr int kDefaultShadowLeafBatch = 26;
+// Sun rays gain from waiting for more lanes.  One rule for both kernels, so
+// that the default pair can be asked for and one tuned value serves both.  Sun
+// rays of the 1024 x 768 nave, one sample, with leaf batches 8, 12, 16, 20, 24,
+// 32 for closest hits: 21.0, 20.1, 18.0, 16.8, 16.5, 19.5 ms with the same value,
+// 17.3, 16.5, 16.4, 16.3, 16.3, 16.3 with this one.
+constexpr int shadow_leaf_batch(int leaf) { return leaf + 10 < 28 ? leaf + 10 : 28; }
 
 // Launchers (rt_kernels.cu).
 struct LaunchCfg {
@@ -277,7 +282,7 @@ struct LaunchCfg {
                 // 3 = leaf batching
   bool sort_rays;  // reorder the vertex >= 2 and sun-ray queues by cell (needs b.rperm)
   int leaf_min;  // lanes waiting at a leaf that start a leaf phase: closest hits
-  int shadow_leaf;  // ... sun rays
+  int shadow_leaf;  // ... sun rays (shadow_leaf_batch)
   int trace_steps, trace_refill;    // closest hit: steps between refill checks, refill threshold
   int shadow_steps, shadow_refill;  // sun rays: the same
 };

@@ -144,7 +144,7 @@ extern "C" rt_status rt_render_static(rt_ctx* c, const rt_camera* cams, uint32_t
   lc.record = false;
   lc.variant = 0;
   lc.leaf_min = kDefaultLeafBatch;
-  lc.shadow_leaf = kDefaultShadowLeafBatch;
+  lc.shadow_leaf = shadow_leaf_batch(lc.leaf_min);
   lc.sort_rays = false;  // the static scratch holds no sort buffers; ray order changes no result
   lc.trace_steps = kDefaultTraceSteps;
   lc.trace_refill = kDefaultTraceRefill;
