@@ -214,9 +214,14 @@ constexpr uint32_t kRayRows = 7;
 // rows of a sun ray behind those: direction, contribution, path id and flags
 constexpr uint32_t kRowDir = 7, kRowContrib = 10, kRowBits = 11, kSunRows = 12;
 
+// FTZ: for unit directions (the paths' own).  A caller's direction past 2^126
+// has a reciprocal below the normal range, and 0 in its place would let the
+// ray enter every box, the empty ones too.
+template <bool FTZ>
 __device__ __forceinline__ float rcp_approx(float x) {
   float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  if (FTZ) asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  else asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
 __device__ __forceinline__ float max3f(float a, float b, float c) {
@@ -236,9 +241,9 @@ template <bool FMA>
 __device__ __forceinline__ void ray4_init(Ray4& r, const RayRows& rows, float3 o, float3 d) {
   rows.put(ray_prep(o, d));
   const float tiny = 1e-20f;
-  r.inv.x = rcp_approx(fabsf(d.x) > tiny ? d.x : copysignf(tiny, d.x));
-  r.inv.y = rcp_approx(fabsf(d.y) > tiny ? d.y : copysignf(tiny, d.y));
-  r.inv.z = rcp_approx(fabsf(d.z) > tiny ? d.z : copysignf(tiny, d.z));
+  r.inv.x = rcp_approx<FMA>(fabsf(d.x) > tiny ? d.x : copysignf(tiny, d.x));
+  r.inv.y = rcp_approx<FMA>(fabsf(d.y) > tiny ? d.y : copysignf(tiny, d.y));
+  r.inv.z = rcp_approx<FMA>(fabsf(d.z) > tiny ? d.z : copysignf(tiny, d.z));
   r.oinv = FMA ? make_float3(o.x * r.inv.x, o.y * r.inv.y, o.z * r.inv.z) : o;
   r.ainv = make_float3(fabsf(r.inv.x), fabsf(r.inv.y), fabsf(r.inv.z));
   r.best_t = INFINITY;
