@@ -475,20 +475,25 @@ def run_photon_mse(args):
 STAGES = ["camera", "closest_hit", "shade_nee", "sun_rays", "xyz", "guide", "train"]
 
 
-def trace_roofline(R, counts, ms_trace, n_trace, ext_rays, prof_ok_traffic=None):
+# bytes a visit reads per child slot of the four-wide tree: a quarter of its 96-byte node
+NODE4_SLOT_BYTES = 24.0
+
+
+def trace_roofline(R, counts, ms_trace, n_trace, ext_rays, prof_ok_traffic=None, slot_bytes=32.0):
     """Roofline of the closest-hit kernel: algorithmic bytes per ray (child
-    slots and triangles tested, from a counting pass, plus the ray and its
-    hit record) times rays per launch over the launch's device time."""
+    slots of slot_bytes each and triangles tested, from a counting pass, plus
+    the ray and its hit record) times rays per launch over the launch's
+    device time."""
     ext_nodes = counts["nodes_visited"] / max(counts["ext_rays"], 1)
     ext_tris = counts["tris_tested"] / max(counts["ext_rays"], 1)
     l2_gbs = R.probe_l2()
     launch_ms = ms_trace / max(n_trace, 1)
     rays_per_launch = ext_rays / max(n_trace, 1)
-    bytes_per_ray = ext_nodes * 32.0 + ext_tris * 48.0 + 32.0 + 8.0
+    bytes_per_ray = ext_nodes * slot_bytes + ext_tris * 48.0 + 32.0 + 8.0
     achieved = rays_per_launch * bytes_per_ray / (launch_ms * 1e-3) / 1e9
     traffic = prof_ok_traffic * rays_per_launch if prof_ok_traffic is not None else None
     return {
-        "kernel": "k_trace (closest hit)", "bound": "l2", "achieved": achieved, "peak": l2_gbs, "unit": "GB/s",
+        "kernel": "k_trace4 (closest hit)", "bound": "l2", "achieved": achieved, "peak": l2_gbs, "unit": "GB/s",
         "frac": achieved / l2_gbs if l2_gbs > 0 else None, "traffic": traffic,
         "peak_source": "L2 streaming-read probe (rt_probe_l2, 48 MiB x 50) measured in this run",
         "hbm_peak_measured": HBM_PEAK, "frac_of_hbm": achieved / HBM_PEAK,
@@ -539,7 +544,7 @@ def nave_subrecord(R, dev, steps=3):
     torch.cuda.synchronize(dev)
     R.set_timing(False)
     ms = e0.elapsed_time(e1) / steps
-    roof = trace_roofline(R, counts, ms_trace, n_trace, ext_rays)
+    roof = trace_roofline(R, counts, ms_trace, n_trace, ext_rays, slot_bytes=NODE4_SLOT_BYTES)
     roof["stage_ms_per_step"] = dict(zip(STAGES, [m / steps for m in stage]))
     return {"workload": NAVE_WORKLOAD, "value": wl.n_paths / (ms * 1e-3), "unit": UNIT, "ms_per_step": ms,
             "steps": steps, "paths_per_step": wl.n_paths, "triangles": int(wl.scene.n_tris), "roofline": roof}
@@ -655,7 +660,7 @@ def main():
     traffic_per_ray = None
     if prof.get("kernel_sources_sha") == kernel_hash() and "dram_bytes_per_ray" in prof:
         traffic_per_ray = float(prof["dram_bytes_per_ray"])
-    roof = trace_roofline(R, counts, ms_trace, n_trace, ext_rays, traffic_per_ray)
+    roof = trace_roofline(R, counts, ms_trace, n_trace, ext_rays, traffic_per_ray, NODE4_SLOT_BYTES)
     roof["stage_ms_per_step"] = dict(zip(STAGES, [m / args.steps for m in stage_ms]))
     roof["sun_rays_per_step"] = counts["shadow_rays"]
     if traffic_per_ray is not None:
@@ -692,7 +697,7 @@ def main():
                 "guide": f"8-lobe vMF MLP guide, one-sample MIS alpha 0.7, guide depth 2, trained online in every "
                          f"pass (every {GUIDE_COLLECT}th path, {GUIDE_STEPS} Adam steps per wave)",
                 "xyz": "f32",
-                "l2": "inputs larger than L2: 2M-triangle BVH and triangles (about 0.3 GB), 1.1 GB of wave queues "
+                "l2": "inputs larger than L2: 2M-triangle BVH and triangles (about 0.2 GB), 1.5 GB of wave queues "
                       "and an 8.2 GB FP64 spectral image per step",
                 "partition": ("each rank renders its band sub-domain of every pass; XYZ partials reduced to rank 0 "
                               "over NCCL" if bands_split else
