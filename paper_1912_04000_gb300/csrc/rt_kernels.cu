@@ -2,19 +2,21 @@
 //
 // One wave holds up to C spectral paths (view, pixel, sample, band).  For each
 // vertex k = 1..depth the host enqueues three kernels:
-//   k_trace  - closest hit of every queued ray (four-wide BVH by default; the
-//              binary, eight-wide and 8-bit-quantised trees as options;
+//   k_trace4 - closest hit of every queued ray over the four-wide BVH (k_trace:
+//              the binary, eight-wide and 8-bit-quantised trees, options;
 //              watertight FP32 test), persistent warps refilling idle lanes
 //              from the queue, leaf batching;
 //   k_shade  - material event at the hit (section 4: Eq. 2 by cosine sampling
 //              for stone, thin-glass/conductor Fresnel events with the complex
 //              index of Eq. 1), next-event estimate of the sun cone (Eq. 3),
 //              continuation ray appended to the next queue;
-//   k_shadow - transmittance of the sun rays (0 behind stone, product of the
-//              thin-glass T_s otherwise), added to the path's radiance.
-// Each path owns one output slot (pixel, band) in the wave, so the FP64
-// accumulation into the spectral image needs no atomics: different samples
-// of a slot are in different waves, which run in sample order.
+//   k_shadow4 - transmittance of the sun rays (0 behind stone, product of the
+//              thin-glass T_s otherwise), added to the path's radiance
+//              (k_shadow: over the binary BVH).
+// The FP64 accumulation into the spectral image needs no atomics: in a wave of
+// one sample or less each path owns its output slot (pixel, band), and waves
+// run in sample order; in a wave of several samples paths leave their radiance
+// in the wave and k_resolve adds it up per slot, in sample order.
 #include <algorithm>
 #include <cstdio>
 #include <type_traits>
@@ -38,15 +40,16 @@ namespace {
 // which covers the rounding of o * inv; the entry distance is shortened by
 // kNearMargin for the relative rounding of both distances.
 // ---------------------------------------------------------------------------
-// Entry distances are shortened by 2^-21 (8 of u = 2^-24) before they are
-// compared with exit and hit distances, at the box test and, as the stacks
-// hold them shortened, when an entry is popped: of an entry distance t the
-// padding leaves up to 4 u t uncovered (2 by the four-wide kernels' approximate
-// reciprocal, 1 by each rounding after it), the other 4 u t are the hit's.
-// Entries popped by the unshortened distance dropped boxes that held a hit at
-// an equal or rounding-nearer distance.
-constexpr float kNearMargin = 1.0f - 0x1p-21f;
-
+// Entry distances are shortened before they are compared with exit and hit
+// distances, at the box test and, as the stacks hold them shortened, when an
+// entry is popped.  In units of u = 2^-24 of an entry distance, the padding
+// leaves uncovered 4 (2 of the four-wide kernels' approximate reciprocal, 1 of
+// each rounding after it), and 5 from any origin, whose distance the padding
+// does not relate to; the exit distance has the same, and a hit's distance the
+// roundings of the triangle test.  Entries popped by the unshortened distance
+// dropped boxes that held a hit at an equal or rounding-nearer distance.
+constexpr float kNearMargin = 1.0f - 0x1p-21f;     // 8 u
+constexpr float kNearMarginAny = 1.0f - 0x1p-20f;  // 16 u: four-wide nodes, any origin
 struct Trav {
   RayW rw;
   float3 inv, oinv;
@@ -256,7 +259,10 @@ __device__ __forceinline__ void ray4_init(Ray4& r, const RayRows& rows, float3 o
 // extent h.  FMA: the rounding of (c - o) / d moves a plane by at most
 // 2^-24 (|o| + |c - o|), within the 2^-22 (max |coordinate| + eps) by which
 // every box is padded, for origins inside the scene bounds.  Otherwise (any
-// origin) from the two planes.
+// origin) the difference first: 4 operations, as many; from the two planes, 8
+// with the selects by the ray's sign, a photon pass of the nave took 1.51 ms
+// (disk) and 8.70 (portals), this way 1.38 and 7.77; a million closest hits
+// 0.297 and 0.262.
 template <bool FMA>
 __device__ __forceinline__ void slab4(float c, float h, float inv, float ainv, float oinv, float& tn, float& tf) {
   if (FMA) {
@@ -264,10 +270,9 @@ __device__ __forceinline__ void slab4(float c, float h, float inv, float ainv, f
     tn = fmaf(-h, ainv, tc);
     tf = fmaf(h, ainv, tc);
   } else {
-    const float t0 = __fmul_rn(__fsub_rn(__fsub_rn(c, h), oinv), inv);
-    const float t1 = __fmul_rn(__fsub_rn(__fadd_rn(c, h), oinv), inv);
-    tn = inv < 0.0f ? t1 : t0;
-    tf = inv < 0.0f ? t0 : t1;
+    const float tc = __fmul_rn(__fsub_rn(c, oinv), inv);
+    tn = fmaf(-h, ainv, tc);
+    tf = fmaf(h, ainv, tc);
   }
 }
 
@@ -284,7 +289,7 @@ __device__ __forceinline__ float child4(const Ray4& r, float cx, float hx, float
   slab4<FMA>(cx, hx, r.inv.x, r.ainv.x, r.oinv.x, nx, fx);
   slab4<FMA>(cy, hy, r.inv.y, r.ainv.y, r.oinv.y, ny, fy);
   slab4<FMA>(cz, hz, r.inv.z, r.ainv.z, r.oinv.z, nz, fz);
-  const float tn = kNearMargin * max3f(nx, ny, fmaxf(nz, 0.0f));
+  const float tn = (FMA ? kNearMargin : kNearMarginAny) * max3f(nx, ny, fmaxf(nz, 0.0f));
   const float tf = min3f(fx, fy, fminf(fz, tmax));
   return tn <= tf ? tn : INFINITY;
 }
@@ -2464,7 +2469,7 @@ void launch_wave(const LaunchCfg& lcfg, const DevScene& S, const DevSpectra& P, 
     // vertex 1 starts at the cameras: where one lies outside the scene bounds,
     // the box test for any origin; later origins are surface points inside the
     // padded bounds (all closest hits of 1024 x 768 x 81 bands x 2 samples in
-    // the 98k-triangle nave: 122.2 ms, with the general test at vertex 1 124.6)
+    // the nave: 122.2 ms, with the general test at vertex 1 124.6)
     launch_trace(lc, k == 1 && !lc.cams_inside, S, qin, b, k, st);
     if (tm) tm->end(STG_TRACE, st);
     if (tm) tm->begin(STG_SHADE, st);

@@ -38,17 +38,18 @@ def load(R, verts, tris, builder):
                               box.mat_thickness[:1].copy()), builder)
 
 
+@pytest.mark.parametrize("distance", [1, 100])
 @pytest.mark.parametrize("builder", [0, 1, 2])
-def test_shared_edges_of_a_far_wall(builder):
+def test_shared_edges_of_a_far_wall(builder, distance):
     from paper_1912_04000_gb300.renderer import Renderer
 
     R = Renderer(0)
     rng = np.random.default_rng(7)
     verts, tris, cls, x, y = wall(rng, 64)
-    # rays from the other half of the scene at points of the grid lines, of
-    # lengths that give every rounding of the reciprocals
+    # rays from the other half of the scene, and from far outside it, at points
+    # of the grid lines, of lengths that give every rounding of the reciprocals
     m = 1 << 20
-    o = rng.uniform(-M, M, (m, 3)).astype(np.float32)
+    o = rng.uniform(-M * distance, M * distance, (m, 3)).astype(np.float32)
     o[:, 2] = -np.abs(o[:, 2])
     to = rng.uniform(-M, M, (m, 3)).astype(np.float32)
     to[:, 2] = M
