@@ -31,7 +31,7 @@ def test_replay_after_the_scene_changed(change):
     before = render(True)
     assert all(torch.equal(a, b) for a, b in zip(before, render(False)))
     if change == "sun":
-        sun = scenes.sun_direction(55.0, 190.0).astype(np.float32)
+        sun = scenes.sun_direction(55.0, 190.0)
         R.set_spectra(dataclasses.replace(wl.spectra, sun_dir=sun, sun_half_angle=0.1))
     elif change == "scene":
         verts = wl.scene.verts.copy()
