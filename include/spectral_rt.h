@@ -384,7 +384,8 @@ rt_status rt_guide_get_params(rt_ctx* ctx, float* grid, float* W);
  * record's omega, for n records rec_dev [n][12] (device, 16-byte aligned). */
 rt_status rt_guide_eval(rt_ctx* ctx, const float* rec_dev, uint64_t n, float* Y_dev, float* q_dev);
 /* Loss and gradients without an update: *loss (host), dgrid_dev and dW_dev
- * (device, FP32, sizes as the parameters; either may be NULL). */
+ * (device, FP32, sizes as the parameters; either may be NULL; after an error
+ * their contents are undefined). */
 rt_status rt_guide_grad(rt_ctx* ctx, const float* rec_dev, uint64_t n, float* loss, float* dgrid_dev, float* dW_dev);
 /* One Adam step on a batch of records; *loss (host, may be NULL) before the step. */
 rt_status rt_guide_train_step(rt_ctx* ctx, const float* rec_dev, uint64_t n, float* loss);

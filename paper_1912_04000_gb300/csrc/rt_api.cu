@@ -24,8 +24,6 @@ struct rt_ctx {
   // diagnostic limits (rt_set_limits; 0 = off): ray-queue capacity, traversal
   // steps per ray, and the countdown to an injected CUDA failure
   uint32_t lim_queue = 0, lim_steps = 0, fail_countdown = 0;
-  int occ_trace = 0;
-  int occ_shade = 0;
   // scene
   float4* d_nodes = nullptr;
   uint32_t* d_nodes4 = nullptr;  // kNode4Words words per node
@@ -95,7 +93,7 @@ struct rt_ctx {
     bool init = false;
     rt_guide_config cfg{};
     float *grid = nullptr, *W = nullptr, *mg = nullptr, *vg = nullptr, *mW = nullptr, *vW = nullptr;
-    float *dgrid = nullptr, *dW = nullptr, *scratch = nullptr;  // scratch: wsum, loss
+    float *dgrid = nullptr, *dW = nullptr, *scratch = nullptr;  // scratch: loss at 1, per-chunk words from 16
     float* dWpart = nullptr;  // per-CTA partial weight gradients, sms x weights
     void* pack = nullptr;
     uint64_t n_grid = 0;
@@ -968,8 +966,8 @@ static rt_status render_impl(rt_ctx* c, const rt_camera* cams, uint32_t n_cams, 
   rt_render_opts o{};
   if (opts) o = *opts;
   if (o.xyz_mode > 2) return fail(c, RT_ERR_ARG, "rt_render: unknown xyz_mode");
-  if (o.xyz_mode != 2 && band_count > kXyzMaxBandsTc)
-    return fail(c, RT_ERR_ARG, "rt_render: tensor-core XYZ takes at most 192 bands (use RT_XYZ_FP64)");
+  if (o.xyz_mode != 2 && band_count > kXyzMaxBands)
+    return fail(c, RT_ERR_ARG, "rt_render: XYZ in FP32 or BF16 takes at most 192 bands (use RT_XYZ_FP64)");
   if (o.trace_variant > 5) return fail(c, RT_ERR_ARG, "rt_render: unknown trace_variant");
   if (o.trace_variant == 5 && !c->d_nodes4q)
     return fail(c, RT_ERR_ARG, "rt_render: the quantised tree needs a host-built BVH (builder 0 or 2)");
@@ -1376,8 +1374,8 @@ rt_status rt_xyz(rt_ctx* c, const double* spectral_dev, uint64_t n_pixels, uint3
   if (!spectral_dev || !xyz_dev || spp == 0 || band_count == 0 || band_first + band_count > c->sp.n_bands ||
       mode > 2)
     return fail(c, RT_ERR_ARG, "rt_xyz: bad argument");
-  if (mode != 2 && band_count > kXyzMaxBandsTc)
-    return fail(c, RT_ERR_ARG, "rt_xyz: tensor-core XYZ takes at most 192 bands (use RT_XYZ_FP64)");
+  if (mode != 2 && band_count > kXyzMaxBands)
+    return fail(c, RT_ERR_ARG, "rt_xyz: XYZ in FP32 or BF16 takes at most 192 bands (use RT_XYZ_FP64)");
   if (((uintptr_t)spectral_dev & 15u) != 0) return fail(c, RT_ERR_ARG, "rt_xyz: spectral_dev must be 16-byte aligned");
   if (n_pixels == 0) return RT_OK;
   cudaSetDevice(c->device);
@@ -1951,8 +1949,8 @@ rt_status rt_render_photons(rt_ctx* c, const rt_camera* cams, uint32_t n_cams, u
   if (hb < 8 || hb > 20) return fail(c, RT_ERR_ARG, "rt_render_photons: log2_cells is 8..20");
   if (o.xyz_mode > 2) return fail(c, RT_ERR_ARG, "rt_render_photons: unknown xyz_mode");
   if (o.emission > 1) return fail(c, RT_ERR_ARG, "rt_render_photons: emission is 0 (disk) or 1 (portals)");
-  if (o.xyz_mode != 2 && band_count > kXyzMaxBandsTc)
-    return fail(c, RT_ERR_ARG, "rt_render_photons: tensor-core XYZ takes at most 192 bands (use RT_XYZ_FP64)");
+  if (o.xyz_mode != 2 && band_count > kXyzMaxBands)
+    return fail(c, RT_ERR_ARG, "rt_render_photons: XYZ in FP32 or BF16 takes at most 192 bands (use RT_XYZ_FP64)");
   if (!(c->cos_max_d > std::cos(1.0)))
     return fail(c, RT_ERR_ARG, "rt_render_photons: photon emission needs a sun half angle below 1 rad");
   if ((o.probe_map_dev != nullptr) != (o.probe_L_dev != nullptr) ||

@@ -420,10 +420,13 @@ __device__ __forceinline__ void encode_levels(const GuideDev& g, const uint32_t*
 // k_guide_count counts the weighted records of each chunk of the batch, a CTA
 // takes its even share of them, in batch order, and compacts their indices
 // into full tiles.
-// Bound by the requests to L2: 64 gathers and 64 adds of 16 bytes per record,
-// 6.4 million for 52,400 weighted records of 524,288, in two bursts per tile;
-// 105 us (126 with two threads per record and equal parts of the batch, whose
-// fullest parts took a fourth tile).
+// Bound by latency: the operand tiles (216 KB) leave room for one CTA per SM, a
+// quarter of the warps, and in each tile the gathers, the chain of MMAs and
+// barriers and the adds follow one another (10.7 long-scoreboard stalls per
+// issue; no unit above a quarter of its peak: L2 15%, L1 21%, issue 15%).  64
+// gathers and 64 adds of 16 bytes per record, 6.4 million for 52,400 weighted
+// records of 524,288: 105 us (126 with two threads per record and equal parts
+// of the batch, whose fullest parts took a fourth tile).
 // Weight gradients dW_l = H_{l-1}^T dZ_l use A' = [H_{l-1}^T; 0] (M = 128)
 // and B' = dZ_l^T, both made from the K-major activation tiles by 8 x 8
 // transposes (ldmatrix / stmatrix.trans), and accumulate in TMEM over all

@@ -31,7 +31,7 @@ constexpr uint32_t kMaxWave = 1u << kPidBits;
 // only widens it; then the children packed as ref << 3 | count:
 //   {cx[4], hx01, hx23, hy01, hy23} {cy[4], hz01, hz23, 0, 0} {cz[4], child[4]}
 // An empty child has a large negative half extent.  Sectors per visit decide
-// the traversal's load on L1 (see trav_interior4).
+// the traversal's load on L1 (see interior4).
 constexpr uint32_t kNode4Bytes = 96, kNode4Words = 24;
 constexpr uint32_t kEmptyHalf = 0xFF7Fu;  // BF16 of -3.4e38
 
@@ -326,9 +326,9 @@ struct XyzWeights {
   uint32_t band_count;
   uint32_t kpad;           // band_count rounded up to 16
 };
-// Tensor-core modes keep all K-slices of a 128-pixel tile in shared memory:
-// at most kXyzMaxBandsTc bands.
-constexpr uint32_t kXyzMaxBandsTc = 192;
+// The FP32 and BF16 modes keep stages of 32 whole rows, or all K-slices of a
+// 128-pixel tile, in shared memory: at most kXyzMaxBands bands.
+constexpr uint32_t kXyzMaxBands = 192;
 void launch_xyz(const double* spectral, uint64_t n_pixels, const XyzWeights& w, uint32_t spp, int mode, float* xyz,
                 cudaStream_t st, uint32_t* status, int sms);
 

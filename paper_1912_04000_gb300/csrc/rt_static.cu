@@ -92,8 +92,8 @@ extern "C" rt_status rt_render_static(rt_ctx* c, const rt_camera* cams, uint32_t
   if (depth == 0 || depth > (uint32_t)kMaxDepth)
     return err(c, RT_ERR_ARG, "rt_render_static: depth must be 1..64 (counter rows in the static array)");
   if (xyz_mode > 2) return err(c, RT_ERR_ARG, "rt_render_static: unknown xyz_mode");
-  if (xyz_mode != 2 && band_count > kXyzMaxBandsTc)
-    return err(c, RT_ERR_ARG, "rt_render_static: tensor-core XYZ takes at most 192 bands (use RT_XYZ_FP64)");
+  if (xyz_mode != 2 && band_count > kXyzMaxBands)
+    return err(c, RT_ERR_ARG, "rt_render_static: XYZ in FP32 or BF16 takes at most 192 bands (use RT_XYZ_FP64)");
   if (((uintptr_t)spectral_dev & 15u) != 0)
     return err(c, RT_ERR_ARG, "rt_render_static: spectral_dev must be 16-byte aligned");
   uint64_t npix = 0;
